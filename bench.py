@@ -288,7 +288,7 @@ def kernel_bytes(fam: str, n: int, ld: int, nnz: int, m: int, wR: int, wD: int, 
 
 
 # sources that define the single-instance streaming kernels (their device code)
-KERNEL_SOURCES = ("common.cuh", "dfloat.cuh", "kernels.cuh", "launch.cuh", "launch_decl.h",
+KERNEL_SOURCES = ("common.cuh", "dfloat.cuh", "rows.cuh", "kernels.cuh", "launch.cuh", "launch_decl.h",
                   "kern_mixed.cu")
 
 

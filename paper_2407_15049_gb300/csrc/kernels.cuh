@@ -7,236 +7,10 @@
 
 #include <type_traits>
 #include "common.cuh"
+#include "rows.cuh"
+#include "cons.cuh"
 
 namespace lorads {
-
-// ------------------------------------------------------------------ problem arrays
-struct ProbDev {
-    int64_t n, m;
-    // C: full symmetric CSR
-    const int64_t* c_rowptr;
-    const int32_t* c_col;
-    const double* c_val;
-    const float* c_val32;
-    const dfloat* c_valdf;
-    // diagonal constraints by row: constraint index (-1: none) and coefficient
-    const int32_t* dk;
-    const double* da;
-    const float* da32;          // float and double-float mirrors of da and b for the
-    const dfloat* da_df;        // FP32-unit paths (no per-row FP64 there)
-    const dfloat* b_df;
-    // off-diagonal constraints as a symmetric pattern: slot -> (column, constraint, coef)
-    const int64_t* a_rowptr;
-    const int32_t* a_col;
-    const int32_t* a_k;
-    const double* a_a;
-    // constraint list, fused diagonal constraints first: triplets (row <= col, coef) in
-    // list order and the constraint of each list position.  k_ptr (general form,
-    // constraints with several triplets): position q owns triplets k_ptr[q]..k_ptr[q+1]-1;
-    // null: position q is triplet q.
-    const int32_t* k_row;
-    const int32_t* k_col;
-    const double* k_a;
-    const int32_t* k_id;
-    const int64_t* k_ptr;
-    int64_t m_diag, m_off;
-    const double* b;
-    // double-float mirrors of the constraint coefficients (list order and pattern
-    // order) for the FP32-unit paths; may be null for FP64 callers
-    const dfloat* k_adf;
-    const dfloat* a_adf;
-};
-
-// ------------------------------------------------------------------ gating
-// Kernels of the captured iteration graph check the control block first and
-// return at once when the current phase does not need them.
-enum { PH_ALWAYS = 0, PH_INNER = 1, PH_STEP = 2, PH_OUTER = 3 };
-
-__device__ __forceinline__ bool gated_off(const Ctrl* g, int ph) {
-    if (g == nullptr || ph == PH_ALWAYS) return false;
-    if (g->solve_done | g->pause) return true;
-    if (ph == PH_OUTER) return g->phase != PHASE_OUTER;
-    if (g->phase != PHASE_INNER) return true;
-    if (ph == PH_STEP) return g->step_ok == 0;
-    return false;
-}
-
-template <typename T>
-using arith_t = typename Arith<T>::type;
-template <typename T>
-using A_of_t = arith_t<T>;
-
-// precision rank of an arithmetic type: float < double-float < double
-template <typename T> struct PrecRank;
-template <> struct PrecRank<float> { static constexpr int v = 0; };
-template <> struct PrecRank<dfloat> { static constexpr int v = 1; };
-template <> struct PrecRank<double> { static constexpr int v = 2; };
-
-template <int R> struct RankType;
-template <> struct RankType<0> { using type = float; };
-template <> struct RankType<1> { using type = dfloat; };
-template <> struct RankType<2> { using type = double; };
-
-// wider of the arithmetic types of two storage types
-template <typename A, typename B>
-using wide_t = typename RankType<(PrecRank<arith_t<A>>::v > PrecRank<arith_t<B>>::v ? PrecRank<arith_t<A>>::v
-                                                                                   : PrecRank<arith_t<B>>::v)>::type;
-
-// partial-sum type: double on the all-FP64 path, double-float otherwise (no FP64 pipe)
-template <typename A, typename B>
-using part_t = std::conditional_t<std::is_same_v<arith_t<A>, double> && std::is_same_v<arith_t<B>, double>,
-                                  double, dfloat>;
-
-// value type of C entries multiplied against rows of type TX
-template <typename TX>
-using cval_t = arith_t<TX>;
-
-template <typename TV> __device__ __forceinline__ const TV* cvals(const ProbDev& p);
-template <> __device__ __forceinline__ const double* cvals<double>(const ProbDev& p) { return p.c_val; }
-template <> __device__ __forceinline__ const float* cvals<float>(const ProbDev& p) { return p.c_val32; }
-template <> __device__ __forceinline__ const dfloat* cvals<dfloat>(const ProbDev& p) { return p.c_valdf; }
-
-// per-row scalar type of the row-update math: double on the FP64 path,
-// otherwise the arithmetic type of R (double-float or float)
-template <typename TR, typename TD>
-using rowscalar_t = std::conditional_t<std::is_same_v<arith_t<TR>, double> && std::is_same_v<arith_t<TD>, double>,
-                                       double, arith_t<TR>>;
-
-template <typename S> __device__ __forceinline__ S ld_scalar(const double* d, const dfloat* df, int64_t k);
-template <> __device__ __forceinline__ double ld_scalar<double>(const double* d, const dfloat*, int64_t k) {
-    return __ldg(d + k);
-}
-template <> __device__ __forceinline__ dfloat ld_scalar<dfloat>(const double*, const dfloat* df, int64_t k) {
-    const float2 v = __ldg(reinterpret_cast<const float2*>(df + k));
-    return dfloat(v.x, v.y);
-}
-template <> __device__ __forceinline__ float ld_scalar<float>(const double*, const dfloat* df, int64_t k) {
-    return __ldg(reinterpret_cast<const float*>(df + k));     // hi part
-}
-
-// type of the per-row z cache (and of the line-search row terms): double on the
-// FP64 path, otherwise the arithmetic type of the direction D
-template <typename TD, typename TR>
-using zrow_t = std::conditional_t<std::is_same_v<part_t<TD, TR>, double>, double, arith_t<TD>>;
-
-// read-only scalar loads
-__device__ __forceinline__ double ldv(const double* p) { return __ldg(p); }
-__device__ __forceinline__ float ldv(const float* p) { return __ldg(p); }
-__device__ __forceinline__ dfloat ldv(const dfloat* p) {
-    const float2 v = __ldg(reinterpret_cast<const float2*>(p));
-    return dfloat(v.x, v.y);
-}
-
-// Warp-uniform row loop: each warp owns 32/L consecutive rows per trip, so the
-// group shuffles below always see the full warp.  Packed groups (`dense`): L may
-// be any width up to 32 (one unit per lane, L = units per row); the warp holds
-// floor(32/L) rows and its last 32 mod L lanes take no row (`live` false), e.g.
-// ld = 24: 5 rows of 6 lanes instead of 4 rows of 8 lanes with 2 idle each.
-struct RowLoop {
-    int L, lig, gw, rows_per_warp, base_lane;
-    bool live;
-    int64_t first, stride;
-    __device__ __forceinline__ RowLoop(int L_, VGrid vg, bool dense = false) : L(L_) {
-        const int lane = threadIdx.x & 31;
-        if (dense) {
-            gw = lane / L;
-            lig = lane - gw * L;
-            rows_per_warp = 32 / L;
-            live = gw < rows_per_warp;
-        } else {
-            lig = threadIdx.x & (L - 1);
-            gw = lane / L;
-            rows_per_warp = 32 / L;
-            live = true;
-        }
-        base_lane = live ? gw * L : 0;
-        const int64_t warp = (vg.bid * (int64_t)blockDim.x + threadIdx.x) >> 5;
-        const int64_t nwarps = ((int64_t)vg.nblk * blockDim.x) >> 5;
-        first = warp * rows_per_warp;
-        stride = nwarps * rows_per_warp;
-    }
-};
-
-// Sum over the L lanes of a packed group, taken in lane order by every lane (the
-// same bits in each lane of the group); all 32 lanes take part in the shuffles.
-__device__ __forceinline__ float shfl_idx(float v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ double shfl_idx(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-__device__ __forceinline__ dfloat shfl_idx(dfloat v, int src) {
-    return dfloat(__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src));
-}
-template <typename V>
-__device__ __forceinline__ V group_sum_packed(V v, int L, int base_lane) {
-    V t = shfl_idx(v, base_lane);
-    for (int k = 1; k < L; ++k) t += shfl_idx(v, base_lane + k);
-    return t;
-}
-
-// Row helpers: lane `lig` of a group of L handles units c*L + lig < Q.
-// Units past Q are zero on load and skipped on store.
-template <typename T, int CPL>
-__device__ __forceinline__ void load_row(Unit<T> (&u)[CPL], const T* base, int64_t row, int ld, int L, int Q, int lig) {
-    const T* p = base + row * (int64_t)ld + lig * 4;
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-        if (c * L + lig < Q) u[c].load(p + c * L * 4);
-        else
-#pragma unroll
-            for (int e = 0; e < 4; ++e) u[c].v[e] = 0;
-    }
-}
-
-template <typename T, int CPL>
-__device__ __forceinline__ void load_row_stream(Unit<T> (&u)[CPL], const T* base, int64_t row, int ld, int L, int Q,
-                                                int lig) {
-    const T* p = base + row * (int64_t)ld + lig * 4;
-#pragma unroll
-    for (int c = 0; c < CPL; ++c) {
-        if (c * L + lig < Q) u[c].load_stream(p + c * L * 4);
-        else
-#pragma unroll
-            for (int e = 0; e < 4; ++e) u[c].v[e] = 0;
-    }
-}
-
-// L2 prefetch (no register, no wait) of one address of global memory.
-__device__ __forceinline__ void prefetch_l2(const void* a) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
-}
-
-// L2 prefetch of the units of `row` that lane `lig` loads: issued one row
-// iteration ahead, it turns the dependent loads of that iteration into L2 hits.
-template <typename T, int CPL>
-__device__ __forceinline__ void prefetch_row(const T* base, int64_t row, int ld, int L, int Q, int lig) {
-    const T* p = base + row * (int64_t)ld + lig * 4;
-#pragma unroll
-    for (int c = 0; c < CPL; ++c)
-        if (c * L + lig < Q) prefetch_l2(p + c * L * 4);
-}
-
-template <typename T, int CPL>
-__device__ __forceinline__ void store_row(const Unit<T> (&u)[CPL], T* base, int64_t row, int ld, int L, int Q, int lig) {
-    T* p = base + row * (int64_t)ld + lig * 4;
-#pragma unroll
-    for (int c = 0; c < CPL; ++c)
-        if (c * L + lig < Q) u[c].store_stream(p + c * L * 4);
-}
-
-template <typename A, typename T1, typename T2, int CPL>
-__device__ __forceinline__ A dot_units(const Unit<T1> (&x)[CPL], const Unit<T2> (&y)[CPL]) {
-    A s = A(0);
-#pragma unroll
-    for (int c = 0; c < CPL; ++c)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s = fma(A(x[c].v[e]), A(y[c].v[e]), s);
-    return s;
-}
-
-// Value an element has once stored as T (bf16 rounds; every other type keeps it).
-template <typename T, typename A>
-__device__ __forceinline__ A as_stored(A v) {
-    if constexpr (std::is_same_v<T, __nv_bfloat16>) return A(__bfloat162float(__float2bfloat16_rn(float(v))));
-    else return v;
-}
 
 // ================================================================== SpMM over C
 // out = C X  (+ the diagonal-constraint part -A*(v) X when v != nullptr),
@@ -245,7 +19,6 @@ __device__ __forceinline__ A as_stored(A v) {
 //            p1 = 2<CD, R>, p2 = <CD, D>, and for diagonal constraints
 //            sum y~ q1, sum y~ q2, sum q1^2, sum q1 q2, sum q2^2
 //   EPI_OBJ: <C X, X> (objective with X = R)
-enum { EPI_NONE = 0, EPI_LS = 1, EPI_OBJ = 2 };
 
 // PF (compile-time, so that the default form carries none of the others' code):
 // 0 none, 1 the next row's bounds and L2 prefetches, 2 also two rows ahead.
@@ -586,301 +359,6 @@ k_spmm_a_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld,
         }
         store_row<TO, CPL>(o, out, i, ld, L, Q, rl.lig);
     }
-}
-
-// ================================================================== constraint pass
-// One group of L lanes per constraint t in [k0, k1) of the ordered list
-// (diagonal constraints first).  With f = 1 (i == j) or 2 (i < j):
-//   CONS_EVAL: out[k] = a (u_i.v_j + [i!=j] u_j.v_i)                  = <A_k, U V^T>
-//   CONS_LS  : z = f a r_i.r_j - b, y~ = y - rho z, q1 = f a (r_i.d_j + d_i.r_j),
-//              q2 = f a d_i.d_j; partials of y~q1, y~q2, q1^2, q1q2, q2^2
-//   CONS_YTIL: out[k] = y~ ;  partial |z|^2
-//   CONS_YUPD: y[k] <- y~ (and its double-float mirror);  partials |z|^2, b^T y_new
-//   CONS_ZZ  : partial |z|^2
-enum { CONS_EVAL = 0, CONS_LS = 1, CONS_YTIL = 2, CONS_YUPD = 3, CONS_ZZ = 4 };
-
-// General form of the constraint pass: list position q is one constraint whose
-// triplets t (i <= j, a) are summed with the weights of the triplet convention:
-//   <A_k, U V^T> = sum_t a (u_i.v_j + [i != j] u_j.v_i),
-// and, with f = 1 (i == j) or 2, z = sum_t f a r_i.r_j - b_k, q1 = sum_t f a
-// (r_i.d_j + d_i.r_j) / (1 + [i == j]) ... written per triplet as in the single-triplet
-// path, then the same per-constraint formulas.  Each lane accumulates its share of
-// every triplet's dots; the group sum follows the triplet loop (no shuffle inside
-// the loop, whose trip count differs between the groups of a warp).
-template <typename TU, typename TV, int CPL, int MODE>
-__device__ __forceinline__ void
-k_cons_general(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const TV* __restrict__ V, int ld, int L,
-               int Q, double* y, void* __restrict__ out, void* zk, dfloat* ydf, const Ctrl* ctrl, double rho_arg,
-               double* __restrict__ part, VGrid vg) {
-    constexpr int NQ = MODE == CONS_LS ? PL_N : PC_N;
-    using PA = part_t<TU, TV>;
-    PA accq[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) accq[q] = PA(0);
-    const double rho = ctrl ? ctrl->rho : rho_arg;
-    const bool same = (const void*)U == (const void*)V;
-    using AU = wide_t<TU, TU>;
-    using AW = wide_t<TU, TV>;
-    using AV = wide_t<TV, TV>;
-    using CS = std::conditional_t<std::is_same_v<PA, double>, double, dfloat>;
-    const CS rho_c = CS(rho);
-    CS* zkc = static_cast<CS*>(zk);
-    RowLoop rl(L, vg);
-    const int64_t cnt = k1 - k0;
-    for (int64_t base = rl.first; base < cnt; base += rl.stride) {
-        const int64_t q = k0 + base + rl.gw;
-        const bool act = q < k1;
-        // per-lane weighted dots: z part (f a u_i.u_j), q1 part, q2 part / EVAL value
-        AU s_z = AU(0);
-        AW s_1 = AW(0);
-        AV s_2 = AV(0);
-        if (act) {
-            const int64_t t0 = __ldg(p.k_ptr + q), t1 = __ldg(p.k_ptr + q + 1);
-            for (int64_t t = t0; t < t1; ++t) {
-                const int i = __ldg(p.k_row + t), j = __ldg(p.k_col + t);
-                const bool dg = i == j;
-                const double a = __ldg(p.k_a + t);
-                const double fa = dg ? a : 2.0 * a;
-                Unit<TU> ui[CPL], uj[CPL];
-                load_row<TU, CPL>(ui, U, i, ld, L, Q, rl.lig);
-                if (!dg) load_row<TU, CPL>(uj, U, j, ld, L, Q, rl.lig);
-                if constexpr (MODE == CONS_EVAL) {
-                    if (same) {
-                        s_z = s_z + AU(fa) * (dg ? dot_units<AU>(ui, ui) : dot_units<AU>(ui, uj));
-                    } else {
-                        Unit<TV> vi[CPL], vj[CPL];
-                        load_row<TV, CPL>(vi, V, i, ld, L, Q, rl.lig);
-                        if (dg) {
-                            s_1 = s_1 + AW(a) * dot_units<AW>(ui, vi);
-                        } else {
-                            load_row<TV, CPL>(vj, V, j, ld, L, Q, rl.lig);
-                            s_1 = s_1 + AW(a) * (dot_units<AW>(ui, vj) + dot_units<AW>(uj, vi));
-                        }
-                    }
-                } else {
-                    if (MODE != CONS_LS || zk == nullptr)
-                        s_z = s_z + AU(fa) * (dg ? dot_units<AU>(ui, ui) : dot_units<AU>(ui, uj));
-                    if constexpr (MODE == CONS_LS) {
-                        Unit<TV> vi[CPL], vj[CPL];
-                        load_row<TV, CPL>(vi, V, i, ld, L, Q, rl.lig);
-                        if (dg) {
-                            const AW d = dot_units<AW>(ui, vi);
-                            s_1 = s_1 + AW(fa) * (d + d);
-                            s_2 = s_2 + AV(fa) * dot_units<AV>(vi, vi);
-                        } else {
-                            load_row<TV, CPL>(vj, V, j, ld, L, Q, rl.lig);
-                            s_1 = s_1 + AW(fa) * (dot_units<AW>(ui, vj) + dot_units<AW>(vi, uj));
-                            s_2 = s_2 + AV(fa) * dot_units<AV>(vi, vj);
-                        }
-                    }
-                }
-            }
-        }
-        s_z = group_sum(s_z, L);
-        s_1 = group_sum(s_1, L);
-        s_2 = group_sum(s_2, L);
-        if (act && rl.lig == 0) {
-            const int k = __ldg(p.k_id + q);
-            if constexpr (MODE == CONS_EVAL) {
-                static_cast<double*>(out)[k] = same ? double(s_z) : double(s_1);
-            } else {
-                CS yk = CS(0.0), bk;
-                if constexpr (MODE != CONS_ZZ) {
-                    if constexpr (std::is_same_v<CS, double>) yk = y[k];
-                    else yk = ydf ? ld_scalar<CS>(y, ydf, k) : CS(y[k]);
-                }
-                if constexpr (std::is_same_v<CS, double>) bk = __ldg(p.b + k);
-                else bk = p.b_df ? ld_scalar<CS>(p.b, p.b_df, k) : CS(__ldg(p.b + k));
-                const CS z = (MODE == CONS_LS && zk != nullptr) ? zkc[k] : CS(s_z) - bk;
-                if constexpr (MODE == CONS_LS) {
-                    const CS yt = yk - rho_c * z;
-                    const CS q1 = CS(s_1);
-                    const CS q2 = CS(s_2);
-                    accq[PL_YQ1] += PA(yt * q1);
-                    accq[PL_YQ2] += PA(yt * q2);
-                    accq[PL_Q1Q1] += PA(q1 * q1);
-                    accq[PL_Q1Q2] += PA(q1 * q2);
-                    accq[PL_Q2Q2] += PA(q2 * q2);
-                } else {
-                    accq[PC_ZZ] += PA(z * z);
-                    if constexpr (MODE == CONS_YTIL) {
-                        static_cast<CS*>(out)[k] = yk - rho_c * z;
-                        if (zk != nullptr) zkc[k] = z;
-                    } else if constexpr (MODE == CONS_YUPD) {
-                        const CS yn = yk - rho_c * z;
-                        y[k] = double(yn);
-                        if constexpr (std::is_same_v<CS, dfloat>) {
-                            if (ydf != nullptr) ydf[k] = yn;
-                        } else {
-                            if (ydf != nullptr) ydf[k] = dfloat(yn);
-                        }
-                        accq[PC_BY] += PA(bk * yn);
-                    }
-                }
-            }
-        }
-    }
-    if constexpr (MODE != CONS_EVAL) block_partials<NQ>(accq, part, vg.pslot);
-}
-
-template <typename TU, typename TV, int CPL, int MODE>
-__device__ __forceinline__ void
-k_cons_body(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const TV* __restrict__ V, int ld, int L, int Q,
-       double* y, void* __restrict__ out, void* zk, dfloat* ydf, const Ctrl* ctrl, double rho_arg,
-       double* __restrict__ part, VGrid vg) {
-    if (p.k_ptr != nullptr) {
-        k_cons_general<TU, TV, CPL, MODE>(p, k0, k1, U, V, ld, L, Q, y, out, zk, ydf, ctrl, rho_arg, part, vg);
-        return;
-    }
-    constexpr int NQ = MODE == CONS_LS ? PL_N : PC_N;
-    using PA = part_t<TU, TV>;
-    PA accq[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) accq[q] = PA(0);
-    const double rho = ctrl ? ctrl->rho : rho_arg;
-    const bool same = (const void*)U == (const void*)V;
-    using AU = wide_t<TU, TU>;
-    using AW = wide_t<TU, TV>;
-    using AV = wide_t<TV, TV>;
-    // per-constraint scalars: double on the all-FP64 path, double-float otherwise
-    // (GB300's FP64 rate is ~1/64 of FP32; conversions run on the FP64 pipe too).
-    // z = A(RR^T)_k - b_k, y~ and the cached z use the same type (zk, out: CS arrays).
-    using CS = std::conditional_t<std::is_same_v<PA, double>, double, dfloat>;
-    const CS rho_c = CS(rho);
-    CS* zkc = static_cast<CS*>(zk);
-    // what each mode gathers besides u_i, u_j
-    constexpr bool NEED_V = MODE == CONS_EVAL || MODE == CONS_LS;
-    // constraints in flight per lane group: the index, coefficient and multiplier
-    // loads and all row gathers of UC constraints are issued before any dot product
-    constexpr int UC = CPL == 1 ? (MODE == CONS_LS || MODE == CONS_EVAL ? 2 : 3) : 1;
-    RowLoop rl(L, vg);
-    const int64_t cnt = k1 - k0;
-    const int64_t step = (int64_t)rl.rows_per_warp;
-    for (int64_t base = rl.first * UC; base < cnt; base += rl.stride * UC) {
-        int64_t t[UC];
-        bool act[UC], diag[UC];
-        int i[UC], j[UC], kid[UC];
-        CS ak[UC], yk[UC], zb[UC];          // coefficient, y_k, and z_k (cached) or b_k
-        Unit<TU> ui[UC][CPL], uj[UC][CPL];
-        Unit<TV> vi[UC][CPL], vj[UC][CPL];
-#pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            t[u] = k0 + base + u * step + rl.gw;
-            act[u] = t[u] < k1;
-            i[u] = act[u] ? __ldg(p.k_row + t[u]) : 0;
-            j[u] = act[u] ? __ldg(p.k_col + t[u]) : 0;
-            if constexpr (MODE == CONS_EVAL || std::is_same_v<CS, double>)
-                ak[u] = act[u] ? CS(__ldg(p.k_a + t[u])) : CS(0.0);
-            else
-                ak[u] = act[u] ? (p.k_adf ? ld_scalar<CS>(p.k_a, p.k_adf, t[u]) : CS(__ldg(p.k_a + t[u]))) : CS(0.0);
-            kid[u] = act[u] ? __ldg(p.k_id + t[u]) : 0;
-            diag[u] = i[u] == j[u];
-        }
-#pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            yk[u] = CS(0.0);
-            zb[u] = CS(0.0);
-            if (!act[u]) continue;
-            if constexpr (MODE != CONS_EVAL) {
-                if constexpr (MODE != CONS_ZZ) {
-                    if constexpr (std::is_same_v<CS, double>) yk[u] = y[kid[u]];
-                    else yk[u] = ydf ? ld_scalar<CS>(y, ydf, kid[u]) : CS(y[kid[u]]);
-                }
-                if (MODE == CONS_LS && zk != nullptr) zb[u] = zkc[kid[u]];
-                else if constexpr (std::is_same_v<CS, double>) zb[u] = __ldg(p.b + kid[u]);
-                else zb[u] = p.b_df ? ld_scalar<CS>(p.b, p.b_df, kid[u]) : CS(__ldg(p.b + kid[u]));
-            }
-            load_row<TU, CPL>(ui[u], U, i[u], ld, L, Q, rl.lig);
-            if (!diag[u]) load_row<TU, CPL>(uj[u], U, j[u], ld, L, Q, rl.lig);
-            if constexpr (NEED_V) {
-                if (!(MODE == CONS_EVAL && same)) {
-                    load_row<TV, CPL>(vi[u], V, i[u], ld, L, Q, rl.lig);
-                    if (!diag[u]) load_row<TV, CPL>(vj[u], V, j[u], ld, L, Q, rl.lig);
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            // dots of the gathered rows; partial per lane, then group sums
-            AU s_uu = AU(0);                  // u_i.u_j (EVAL with U==V, and R-only modes)
-            AW s_uv = AW(0), s_vu = AW(0);    // u_i.v_j, u_j.v_i
-            AV s_vv = AV(0);                  // v_i.v_j
-            if (act[u]) {
-                if constexpr (MODE == CONS_EVAL) {
-                    if (same) {
-                        s_uu = diag[u] ? dot_units<AU>(ui[u], ui[u]) : dot_units<AU>(ui[u], uj[u]);
-                    } else if (diag[u]) {
-                        s_uv = dot_units<AW>(ui[u], vi[u]);
-                    } else {
-                        s_uv = dot_units<AW>(ui[u], vj[u]);
-                        s_vu = dot_units<AW>(uj[u], vi[u]);
-                    }
-                } else {
-                    if (MODE != CONS_LS || zk == nullptr)
-                        s_uu = diag[u] ? dot_units<AU>(ui[u], ui[u]) : dot_units<AU>(ui[u], uj[u]);
-                    if constexpr (MODE == CONS_LS) {
-                        if (diag[u]) {
-                            s_uv = dot_units<AW>(ui[u], vi[u]);
-                            s_vu = s_uv;
-                            s_vv = dot_units<AV>(vi[u], vi[u]);
-                        } else {
-                            s_uv = dot_units<AW>(ui[u], vj[u]);
-                            s_vu = dot_units<AW>(vi[u], uj[u]);
-                            s_vv = dot_units<AV>(vi[u], vj[u]);
-                        }
-                    }
-                }
-            }
-            s_uu = group_sum(s_uu, L);
-            if constexpr (MODE == CONS_EVAL || MODE == CONS_LS) {
-                s_uv = group_sum(s_uv, L);
-                s_vu = group_sum(s_vu, L);
-                s_vv = group_sum(s_vv, L);
-            }
-            if (act[u] && rl.lig == 0) {
-                const int k = kid[u];
-                if constexpr (MODE == CONS_EVAL) {
-                    const double a = double(ak[u]);
-                    const double f = diag[u] ? 1.0 : 2.0;
-                    double val;
-                    if (same) val = f * a * double(s_uu);
-                    else if (diag[u]) val = a * double(s_uv);
-                    else val = a * (double(s_uv) + double(s_vu));
-                    static_cast<double*>(out)[k] = val;
-                } else {
-                    const CS fa = diag[u] ? ak[u] : CS(2.0f) * ak[u];
-                    const CS z = (MODE == CONS_LS && zk != nullptr) ? zb[u] : fa * CS(s_uu) - zb[u];
-                    if constexpr (MODE == CONS_LS) {
-                        const CS yt = yk[u] - rho_c * z;
-                        const CS q1 = fa * (CS(s_uv) + CS(s_vu));
-                        const CS q2 = fa * CS(s_vv);
-                        accq[PL_YQ1] += PA(yt * q1);
-                        accq[PL_YQ2] += PA(yt * q2);
-                        accq[PL_Q1Q1] += PA(q1 * q1);
-                        accq[PL_Q1Q2] += PA(q1 * q2);
-                        accq[PL_Q2Q2] += PA(q2 * q2);
-                    } else {
-                        accq[PC_ZZ] += PA(z * z);
-                        if constexpr (MODE == CONS_YTIL) {
-                            static_cast<CS*>(out)[k] = yk[u] - rho_c * z;
-                            if (zk != nullptr) zkc[k] = z;
-                        } else if constexpr (MODE == CONS_YUPD) {
-                            const CS yn = yk[u] - rho_c * z;
-                            y[k] = double(yn);
-                            if constexpr (std::is_same_v<CS, dfloat>) {
-                                if (ydf != nullptr) ydf[k] = yn;
-                            } else {
-                                if (ydf != nullptr) ydf[k] = dfloat(yn);
-                            }
-                            // b_k: zb holds it (z is recomputed in this mode)
-                            accq[PC_BY] += PA(zb[u] * yn);
-                        }
-                    }
-                }
-            }
-        }
-    }
-    if constexpr (MODE != CONS_EVAL) block_partials<NQ>(accq, part, vg.pslot);
 }
 
 // ================================================================== direction
