@@ -19,6 +19,7 @@
 #include "kernels.cuh"
 #include "launch_decl.h"
 #include "prob_host.h"
+#include "spmm_tile.cuh"
 
 using namespace lorads;
 
@@ -190,6 +191,21 @@ int row_blocks(const lorads_ctx* c, int64_t rows, int L) {
     int64_t b = (rows + per_block - 1) / per_block;
     if (b < 1) b = 1;
     return (int)std::min<int64_t>(b, c->max_blocks);
+}
+
+// Fills the grid of a product over C: the tile kernel where a row has one unit per lane.
+// Returns the blocks launched (those whose partial sums the caller folds).
+template <typename TX, typename TO>
+int plan_spmm(const lorads_ctx* c, SpmmCArgs* a) {
+    if (a->sh.Q <= 32) {
+        const TilePlan t = tile_plan(c->n, a->sh.Q, c->num_sms * tile_blocks<TX, TO>(), tile_threads<TX, TO>());
+        a->nsub = t.nsub;
+        a->blocks = t.blocks;
+    } else {
+        a->nsub = 0;
+        a->blocks = row_blocks(c, c->n, a->sh.L);
+    }
+    return a->blocks;
 }
 
 int flat_blocks(const lorads_ctx* c, int64_t items) {
@@ -476,14 +492,17 @@ extern "C" lorads_status lorads_spmm(lorads_ctx* ctx, const void* R, int32_t r, 
     SpmmAArgs aa{ctx->pd, R, out, ld, sh, v, -1.0, 1, nb, nullptr, PH_ALWAYS, ctx->stream};
     switch (prec) {
         case LORADS_FP64:
+            plan_spmm<double, double>(ctx, &a);
             launch_spmm_c<double, double, double>(a);
             if (v && ctx->m_off) launch_spmm_a<double, double>(aa);
             break;
         case LORADS_FP32:
+            plan_spmm<float, float>(ctx, &a);
             launch_spmm_c<float, float, float>(a);
             if (v && ctx->m_off) launch_spmm_a<float, float>(aa);
             break;
         default:
+            plan_spmm<bf16, float>(ctx, &a);
             launch_spmm_c<bf16, float, bf16>(a);
             if (v && ctx->m_off) launch_spmm_a<bf16, float>(aa);
             break;
@@ -520,7 +539,7 @@ extern "C" lorads_status lorads_linesearch_coeffs(lorads_ctx* ctx, const void* R
         return set_err(ctx, "R, D, y must be device pointers (R, D 16-byte aligned) and a_out non-NULL"),
                LORADS_ERR_INVALID_ARG;
     if (!std::isfinite(rho) || rho < 0) return set_err(ctx, "rho must be finite and >= 0"), LORADS_ERR_INVALID_ARG;
-    const int nb = row_blocks(ctx, ctx->n, sh.L);
+    int nb = 0;
     const int nbc = row_blocks(ctx, std::max<int64_t>(ctx->m_off, 1), sh.L);
     double* pl = part_of(ctx, PART_LS);
     double* pc = part_of(ctx, PART_CONS_LS);
@@ -530,14 +549,17 @@ extern "C" lorads_status lorads_linesearch_coeffs(lorads_ctx* ctx, const void* R
                 pc, nbc, nullptr, PH_ALWAYS, ctx->stream};
     switch (prec) {
         case LORADS_FP64:
+            nb = plan_spmm<double, double>(ctx, &a);
             launch_spmm_c<double, double, double>(a);
             launch_cons<double, double>(ca);
             break;
         case LORADS_FP32:
+            nb = plan_spmm<float, float>(ctx, &a);
             launch_spmm_c<float, float, float>(a);
             launch_cons<float, float>(ca);
             break;
         default:
+            nb = plan_spmm<bf16, float>(ctx, &a);
             launch_spmm_c<bf16, float, bf16>(a);
             launch_cons<bf16, bf16>(ca);
             break;
@@ -563,7 +585,7 @@ struct Driver {
     lorads_ctx* c;
     SolverState& st;
     cudaStream_t s;
-    int nb_rows, nb_ls, nb_flat, nb_off, nb_all;
+    int nb_rows, nb_ls, nb_obj, nb_flat, nb_off, nb_all;
     int64_t nunits;
 
     Driver(lorads_ctx* ctx) : c(ctx), st(ctx->st), s(ctx->solve_stream) { refresh(); }
@@ -571,6 +593,7 @@ struct Driver {
     void refresh() {
         nb_rows = row_blocks(c, c->n, st.sh.L);
         nb_ls = row_blocks(c, c->n, st.sh_ls.L);
+        nb_obj = obj_args(PH_OUTER).blocks;
         nunits = c->n * (int64_t)st.ld / 4;
         nb_flat = flat_blocks(c, nunits);
         nb_off = row_blocks(c, std::max<int64_t>(c->m_off, 1), st.sh.L);
@@ -613,9 +636,14 @@ struct Driver {
         });
     }
 
+    SpmmCArgs obj_args(int ph) const {
+        SpmmCArgs a{c->pd, st.R, st.CR, st.ld, st.sh, nullptr, 1, EPI_OBJ, st.R, st.y, nullptr, nullptr, c->ctrl, 0.0,
+                    part_of(c, PART_OBJ), 0, c->ctrl, ph, s};
+        plan_spmm<TR, TR>(c, &a);
+        return a;
+    }
     void spmm_CR(int ph) {
-        SpmmCArgs a{p(), st.R, st.CR, st.ld, st.sh, nullptr, 1, EPI_OBJ, st.R, st.y, nullptr, nullptr, c->ctrl, 0.0,
-                    part_of(c, PART_OBJ), nb_rows, c->ctrl, ph, s};
+        const SpmmCArgs a = obj_args(ph);
         timed(FAM_SPMM_CR, [&] { launch_spmm_c<TR, TR, TR>(a); });
     }
 
@@ -624,7 +652,7 @@ struct Driver {
         ConsArgs zz{p(), CONS_ZZ, 0, c->m, st.R, st.R, st.ld, st.sh, st.y, nullptr, nullptr, nullptr, c->ctrl, 0.0,
                     part_of(c, PART_CONS), nb_all, c->ctrl, PH_ALWAYS, s};
         timed(FAM_MISC, [&] { launch_cons<TR, TR>(zz); });
-        timed(FAM_MISC, [&] { ctrl_init(s, c->ctrl, part_of(c, PART_CONS), nb_all, part_of(c, PART_OBJ), nb_rows); });
+        timed(FAM_MISC, [&] { ctrl_init(s, c->ctrl, part_of(c, PART_CONS), nb_all, part_of(c, PART_OBJ), nb_obj); });
         outer_gradient(PH_OUTER);
     }
 
@@ -680,7 +708,7 @@ struct Driver {
         timed(FAM_CONS_YUPD, [&] { launch_cons<TR, TR>(yu); });
         spmm_CR(PH_OUTER);
         timed(FAM_OUTER, [&] {
-            ctrl_outer(s, c->ctrl, part_of(c, PART_CONS), nb_all, part_of(c, PART_OBJ), nb_rows);
+            ctrl_outer(s, c->ctrl, part_of(c, PART_CONS), nb_all, part_of(c, PART_OBJ), nb_obj);
         });
         outer_gradient(PH_OUTER);
     }
@@ -1058,13 +1086,14 @@ int64_t admm_enqueue_outer(lorads_ctx* ctx, const AdmmRows& rows) {
     admm_yupd<TR>(rows, a.U, a.V, st.y, st.ydf, a.ac, part_of(ctx, PART_YTIL));
     admm_avg<TR>(rows, a.U, a.V, st.R);
     SpmmCArgs o{ctx->pd, st.R, st.CR, rows.ld, rows.sh, nullptr, 1, EPI_OBJ, st.R, st.y, nullptr, nullptr, nullptr,
-                0.0, part_of(ctx, PART_OBJ), rows.nb_rows, nullptr, PH_ALWAYS, s};
+                0.0, part_of(ctx, PART_OBJ), 0, nullptr, PH_ALWAYS, s};
+    const int nb_obj = plan_spmm<TR, TR>(ctx, &o);
     launch_spmm_c<TR, TR, TR>(o);
     ConsArgs z{ctx->pd, CONS_ZZ, 0, ctx->m, st.R, st.R, rows.ld, rows.sh, nullptr, nullptr, nullptr, nullptr,
                nullptr, 0.0, part_of(ctx, PART_CONS), rows.nb_cons, nullptr, PH_ALWAYS, s};
     launch_cons<TR, TR>(z);
     admm_outer(s, a.ac, part_of(ctx, PART_YTIL), rows.nb_cons, part_of(ctx, PART_CONS), rows.nb_cons,
-               part_of(ctx, PART_OBJ), rows.nb_rows);
+               part_of(ctx, PART_OBJ), nb_obj);
     return 5;
 }
 
@@ -1560,7 +1589,8 @@ lorads_status run_lanczos(lorads_ctx* ctx, const double* ydev, int k, uint64_t s
     lz_scale(s, n, v, lz, sc, nbf);
     for (int j = 0; j < k; ++j) {
         SpmmCArgs a{ctx->pd, v, w, 4, sh, ydev, 1, EPI_NONE, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0,
-                    nullptr, nbr, nullptr, PH_ALWAYS, s};
+                    nullptr, 0, nullptr, PH_ALWAYS, s};
+        plan_spmm<double, double>(ctx, &a);
         launch_spmm_c<double, double, double>(a);
         if (ctx->m_off) {
             SpmmAArgs aa{ctx->pd, v, w, 4, sh, ydev, -1.0, 1, nbr, nullptr, PH_ALWAYS, s};

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "spmm_tile.cuh"
 #include "launch_decl.h"
 
 namespace lorads {
@@ -24,10 +25,23 @@ void launch_spmm_c_one(const SpmmCArgs& a, int L) {
         static_cast<const TR*>(a.R), a.y, a.zrow, a.ydf, a.ctrl, a.rho, a.part, a.gate, a.ph);
 }
 
+template <typename TX, typename TO, typename TR, int EPI>
+void launch_spmm_tile(const SpmmCArgs& a) {
+    k_spmm_tile<TX, TO, TR, EPI><<<a.blocks, tile_threads<TX, TO>(), 0, a.stream>>>(
+        a.p, static_cast<const TX*>(a.X), static_cast<TO*>(a.out), a.ld, a.sh.Q, a.nsub, a.v, a.write_out,
+        static_cast<const TR*>(a.R), a.y, a.rho, a.part, a.gate, a.ph);
+}
+
 // The line-search form takes the prefetch depth (and packed groups) as template
 // arguments; the other epilogues run without prefetch.
 template <typename TX, typename TO, typename TR>
 void launch_spmm_c(const SpmmCArgs& a) {
+    if (a.nsub > 0) {
+        if (a.epi == EPI_LS) launch_spmm_tile<TX, TO, TR, EPI_LS>(a);
+        else if (a.epi == EPI_OBJ) launch_spmm_tile<TX, TO, TR, EPI_OBJ>(a);
+        else launch_spmm_tile<TX, TO, TR, EPI_NONE>(a);
+        return;
+    }
     if (a.epi == EPI_LS && a.dense && packed_rows_gain(a.sh)) {
         if (a.prefetch == 2) launch_spmm_c_one<TX, TO, TR, 1, EPI_LS, true, 2>(a, a.sh.Q);
         else if (a.prefetch == 1) launch_spmm_c_one<TX, TO, TR, 1, EPI_LS, true, 1>(a, a.sh.Q);

@@ -19,6 +19,7 @@ struct SpmmCArgs {
     int prefetch = 0;   // 1: carry the next row's bounds and prefetch its entries and row terms into L2;
                         // 2: also the bounds of the row after next and one neighbour row of the next row
     int dense = 0;      // line-search epilogue: packed row groups of Q lanes (one unit per lane)
+    int nsub = 0;       // > 0: the tile kernel (rows of one unit per lane), row groups a tile
 };
 
 // v: double[m], or double-float[m] when v_df (weights then formed without FP64)

@@ -31,6 +31,7 @@
 #include "control.h"
 #include "kernels.cuh"
 #include "launch_decl.h"
+#include "spmm_tile.cuh"
 
 using namespace lorads;
 
@@ -138,11 +139,18 @@ extern "C" lorads_status lorads_linesearch_coeffs_noalloc(
     p.b = b;
     p.m_diag = 0;
     p.m_off = m;
-    const int nb_rows = capped_blocks(n, sh.L);
+    // the tile kernel: a grid of at most kNoallocBlocks blocks
+    int nsub = 0, nb_rows = capped_blocks(n, sh.L);
+    if (sh.Q <= 32) {
+        const TilePlan t = tile_plan(n, sh.Q, kNoallocBlocks, tile_threads<double, double>());
+        nsub = t.nsub;
+        nb_rows = t.blocks;
+    }
     const int nb_cons = capped_blocks(m, sh.L);
     // p1 = 2<CD, R>, p2 = <CD, D> over C; then the constraint terms; then a1..a4, tau
     SpmmCArgs a{p, D, nullptr, ld, sh, nullptr, 0, EPI_LS, R, y, nullptr, nullptr, nullptr, rho, part_ls,
                 nb_rows, nullptr, PH_ALWAYS, stream};
+    a.nsub = nsub;
     launch_spmm_c<double, double, double>(a);
     ConsArgs ca{p, CONS_LS, 0, m, R, D, ld, sh, const_cast<double*>(y), nullptr, nullptr, nullptr, nullptr, rho,
                 part_cons, nb_cons, nullptr, PH_ALWAYS, stream};

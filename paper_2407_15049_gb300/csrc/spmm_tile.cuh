@@ -1,0 +1,281 @@
+// The SpMM over C for rows of one unit per lane (up to 128 elements): a warp owns a tile of
+// consecutive rows, its lanes in packed groups of Q = ld/4 (one unit each, floor(32/Q) rows
+// at a time, nsub times).
+#pragma once
+
+#include "rows.cuh"
+#include "cons.cuh"
+
+namespace lorads {
+
+constexpr int kTileLaneRows = 192;        // row sums of a tile: rows x Q partials at most
+constexpr int kTileEntries = 160;         // stored entries of a tile held in shared memory
+
+// Threads per block: 8-byte forms take twice the shared memory a warp.
+template <typename TX, typename TO> constexpr int tile_threads() {
+    return sizeof(arith_t<TX>) == 8 || sizeof(arith_t<TO>) == 8 ? 128 : 256;
+}
+// Resident blocks the kernel is compiled for.
+template <typename TX, typename TO> constexpr int tile_blocks() { return tile_threads<TX, TO>() == 128 ? 4 : 3; }
+
+// Row groups a warp takes in turn (nsub) and the grid: one resident wave of warps that walk
+// the tiles; small problems take tiles of one row group, so that every row has its lanes.
+struct TilePlan {
+    int nsub, blocks;
+};
+inline TilePlan tile_plan(int64_t n, int Q, int most_blocks, int threads) {
+    const int rpw = 32 / Q, nw = threads / 32;
+    int most = 32 / rpw;
+    if (most > kTileLaneRows / (rpw * Q)) most = kTileLaneRows / (rpw * Q);
+    int64_t nsub = n / ((int64_t)rpw * most_blocks * nw);
+    nsub = nsub < 1 ? 1 : (nsub > most ? most : nsub);
+    const int64_t tiles = (n + rpw * nsub - 1) / (rpw * nsub);
+    const int64_t blocks = (tiles + nw - 1) / nw;
+    return TilePlan{(int)nsub, (int)(blocks < most_blocks ? blocks : most_blocks)};
+}
+
+// 4 or 8 bytes of global memory to shared memory, without a register.
+template <int BYTES>
+__device__ __forceinline__ void stage_bytes(void* smem, const void* g) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(g), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// out = C X (- A*_diag(v) X), EPI as in k_spmm_c (kernels.cuh); EPI_LS without a cache of z (the
+// line search of a caller's own method).  Why tiles: with one row group at a time every lane of
+// the group loaded the row's bounds, entries and multiplier term for itself, the row sums took
+// shuffles in every lane, and the scalar terms of the line search ran with one lane of the group
+// at work; in FP64 (2 lanes a cycle and SM) they cost as much as the products, and the weight of
+// the diagonal constraint, formed by every lane, more than the float row's multiply-adds.  Here
+//  - the bounds and per-row scalars of the tile are loaded by lane = row (coalesced), the weight
+//    and the line-search scalars formed by lane = row, once per tile;
+//  - the stored entries of the next tile are copied to shared memory (cp.async) while this one
+//    is computed, so that a row's gathers wait on no index load;
+//  - the row sums go through shared memory and are taken by lane = row in lane order.
+// Element sums keep the order of the stored entries.  Measured: line search in FP64, n = 1e6,
+// ld = 20, 5e6 entries: 1437 -> 631 us (346 us of FP64 multiply-adds at two lanes a cycle);
+// double-float C R with the objective, n = 1e6, ld = 24: 840 -> 342 us; float product with a
+// multiplier on a 1000 x 1000 torus, ld = 20: 146 -> 121 us.  The line search of the solve keeps
+// k_spmm_c: its scalars are few in float, and the tile form (24 resident warps instead of 32)
+// took 318 us where k_spmm_c takes 224 (n = 1e6, ld = 24).
+template <typename TX, typename TO, typename TR, int EPI>
+__global__ void __launch_bounds__((tile_threads<TX, TO>()), (tile_blocks<TX, TO>()))
+k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, int Q, int nsub,
+            const double* __restrict__ v, int write_out, const TR* __restrict__ R, const double* __restrict__ y,
+            double rho_arg, double* __restrict__ part, const Ctrl* gate, int ph) {
+    if (gated_off(gate, ph)) return;
+    using A = arith_t<TO>;
+    using TV = cval_t<TX>;
+    using PA = part_t<TO, TR>;
+    using LS = zrow_t<TX, TR>;
+    using AW = wide_t<TR, TX>;
+    using AD = arith_t<TX>;
+    constexpr int NW = tile_threads<TX, TO>() / 32;
+    constexpr int UN = sizeof(AD) == 8 ? 4 : 8;            // gathers in flight per lane
+    constexpr bool kSums = EPI == EPI_LS;
+    __shared__ __align__(16) int s_col[NW][2][kTileEntries];
+    __shared__ __align__(16) TV s_val[NW][2][kTileEntries];
+    __shared__ AD s_rd[NW][kSums ? kTileLaneRows : 1], s_dd[NW][kSums ? kTileLaneRows : 1];
+    __shared__ AW s_rr[NW][kSums ? kTileLaneRows : 1];
+    const TV* __restrict__ cv = cvals<TV>(p);
+    constexpr int NQ = EPI == EPI_LS ? PL_N : (EPI == EPI_OBJ ? PO_N : 1);
+    PA accq[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) accq[q] = PA(0);
+    const LS rho = LS(rho_arg);
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int rpw = 32 / Q, gw = lane / Q, lig = lane - gw * Q;
+    const bool live = gw < rpw;
+    const int rows = rpw * nsub;
+    const int64_t ntiles = (p.n + rows - 1) / rows;
+    const int64_t nwarps = (int64_t)gridDim.x * NW;
+    int64_t t = (int64_t)blockIdx.x * NW + wib;
+
+    // bounds of the lane's row of tile tt (an empty range past the tile's or the matrix's end)
+    auto bounds = [&](int64_t tt, int64_t& s, int64_t& e) {
+        s = e = 0;
+        if (tt < ntiles) {
+            const int64_t r = tt * rows + (lane < rows ? lane : rows);
+            s = __ldg(p.c_rowptr + (r < p.n ? r : p.n));
+            e = lane < rows && r < p.n ? __ldg(p.c_rowptr + r + 1) : s;
+        }
+    };
+    // entries [first, last) of a tile to buffer `buf` (a longer tile is read from global memory)
+    auto stage = [&](int buf, int64_t first, int64_t last) {
+        if (last - first <= kTileEntries)
+            for (int k = lane; k < (int)(last - first); k += 32) {
+                stage_bytes<4>(&s_col[wib][buf][k], p.c_col + first + k);
+                stage_bytes<sizeof(TV)>(&s_val[wib][buf][k], cv + first + k);
+            }
+        stage_commit();
+    };
+    int64_t s_nx, e_nx, first;           // bounds of the next tile's rows; first entry of this one
+    bounds(t, s_nx, e_nx);
+    first = __shfl_sync(0xffffffffu, s_nx, 0);
+    int64_t end = __shfl_sync(0xffffffffu, e_nx, 31);
+    // of the lane's row: its length, and where it starts (in the tile, when that is staged)
+    int my_len = (int)(e_nx - s_nx);
+    bool in_smem = end - first <= kTileEntries;
+    int64_t my_at = in_smem ? s_nx - first : s_nx;
+    int buf = 0;
+    stage(0, first, end);
+    bounds(t + nwarps, s_nx, e_nx);
+    for (; t < ntiles; t += nwarps) {
+        first = __shfl_sync(0xffffffffu, s_nx, 0);
+        end = __shfl_sync(0xffffffffu, e_nx, 31);
+        stage(buf ^ 1, first, end);
+        const int len_nx = (int)(e_nx - s_nx);
+        const bool smem_nx = end - first <= kTileEntries;
+        const int64_t at_nx = smem_nx ? s_nx - first : s_nx;
+        bounds(t + 2 * nwarps, s_nx, e_nx);
+        const int64_t r0 = t * rows;
+        // per-row scalars of lane = row
+        const int64_t my = r0 + lane;
+        const bool own = lane < rows && my < p.n;
+        int kc = -1;
+        A wv = A(0);
+        if (p.dk != nullptr && own) {
+            kc = __ldg(p.dk + my);
+            if (v != nullptr && kc >= 0) wv = A(-__ldg(p.da + my) * __ldg(v + kc));
+        }
+        stage_wait<1>();
+        __syncwarp();
+        const int* sc = s_col[wib][buf];
+        const TV* sv = s_val[wib][buf];
+        const bool diag = v != nullptr && p.dk != nullptr;
+#pragma unroll 1
+        for (int sb = 0; sb < nsub; ++sb) {
+            const int lr = sb * rpw + gw;                  // the group's row of the tile
+            const int64_t i = r0 + lr;
+            const bool act = live && i < p.n;
+            const int src = live ? lr : 0;
+            const int len = __shfl_sync(0xffffffffu, my_len, src);
+            // the row's entries: in shared memory, or where they are (generic addresses)
+            const int64_t at = __shfl_sync(0xffffffffu, my_at, src);
+            const int* rc = in_smem ? sc + (int)at : p.c_col + at;
+            const TV* rv = in_smem ? sv + (int)at : cv + at;
+            LaneDot<A> acc[4];
+            Unit<TX> di;
+            Unit<TR> ri;
+            if (act) {
+                if constexpr (EPI != EPI_NONE) di.load(X + i * (int64_t)ld + lig * 4);
+                if constexpr (EPI == EPI_LS) ri.load_stream(R + i * (int64_t)ld + lig * 4);
+            }
+            for (int k = 0; act && k < len; k += UN) {
+                int j[UN];
+                TV w[UN];
+                Unit<TX> x[UN];
+#pragma unroll
+                for (int u = 0; u < UN; ++u) {
+                    const bool ok = k + u < len;
+                    j[u] = -1;
+                    w[u] = TV(0);
+                    if (ok) {
+                        j[u] = rc[k + u];
+                        w[u] = rv[k + u];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < UN; ++u)
+                    if (j[u] >= 0) x[u].load(X + (int64_t)j[u] * ld + lig * 4);
+#pragma unroll
+                for (int u = 0; u < UN; ++u)
+                    if (j[u] >= 0)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[e].add(A(w[u]), A(x[u].v[e]));
+            }
+            if (diag) {
+                const int kr = __shfl_sync(0xffffffffu, kc, src);
+                const A w = shfl_idx(wv, src);
+                if (act && kr >= 0) {
+                    Unit<TX> xi;
+                    if constexpr (EPI != EPI_NONE) xi = di;
+                    else xi.load(X + i * (int64_t)ld + lig * 4);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[e].add(w, A(xi.v[e]));
+                }
+            }
+            A o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[e] = acc[e].value();
+            if (write_out && act) {
+                Unit<TO> ou;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) ou.v[e] = o[e];
+                ou.store_stream(out + i * (int64_t)ld + lig * 4);
+            }
+            if constexpr (EPI == EPI_OBJ) {
+                if (act) {
+                    LaneDot<A> d;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) d.add(o[e], A(di.v[e]));
+                    accq[PO_CRR] += PA(d.value());
+                }
+            }
+            if constexpr (EPI == EPI_LS) {
+                if (act) {
+                    AD p2 = AD(0);
+                    LaneDot<AD> rd, dd;
+                    LaneDot<AW> p1, rr;
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const AD d = AD(di.v[e]);
+                        p2 = fma(AD(o[e]), d, p2);
+                        rd.add(AD(ri.v[e]), d);
+                        dd.add(d, d);
+                        const AW r = AW(ri.v[e]);
+                        p1.add(AW(o[e]), r);
+                        rr.add(r, r);
+                    }
+                    accq[PL_P2] += p2;
+                    s_rd[wib][lr * Q + lig] = rd.value();
+                    s_dd[wib][lr * Q + lig] = dd.value();
+                    accq[PL_P1] += PA(AW(2) * p1.value());
+                    s_rr[wib][lr * Q + lig] = rr.value();
+                }
+            }
+        }
+        __syncwarp();
+        if constexpr (EPI == EPI_LS) {
+            if (kc >= 0) {
+                AD t_rd = s_rd[wib][lane * Q], t_dd = s_dd[wib][lane * Q];
+                AW t_rr = s_rr[wib][lane * Q];
+                for (int q = 1; q < Q; ++q) {
+                    t_rd += s_rd[wib][lane * Q + q];
+                    t_dd += s_dd[wib][lane * Q + q];
+                    t_rr += s_rr[wib][lane * Q + q];
+                }
+                LS a, z, yv;
+                if constexpr (std::is_same_v<LS, double>) {
+                    a = __ldg(p.da + my);
+                    z = a * double(t_rr) - __ldg(p.b + kc);
+                    yv = __ldg(y + kc);
+                } else {
+                    a = ld_scalar<LS>(p.da, p.da_df, my);
+                    z = LS(dfloat(t_rr) * ld_scalar<dfloat>(p.da, p.da_df, my) - ld_scalar<dfloat>(p.b, p.b_df, kc));
+                    yv = LS(__ldg(y + kc));
+                }
+                const LS yt = yv - rho * z;
+                const LS q1 = LS(2) * a * LS(t_rd);
+                const LS q2 = a * LS(t_dd);
+                accq[PL_YQ1] += PA(yt * q1);
+                accq[PL_YQ2] += PA(yt * q2);
+                accq[PL_Q1Q1] += PA(q1 * q1);
+                accq[PL_Q1Q2] += PA(q1 * q2);
+                accq[PL_Q2Q2] += PA(q2 * q2);
+            }
+            __syncwarp();                                  // the sums have been read
+        }
+        my_len = len_nx;
+        my_at = at_nx;
+        in_smem = smem_nx;
+        buf ^= 1;
+    }
+    stage_wait<0>();
+    if constexpr (EPI != EPI_NONE) block_partials<NQ>(accq, part, (int)blockIdx.x);
+}
+
+}  // namespace lorads
