@@ -194,10 +194,6 @@ template <typename T> struct Arith { using type = T; };
 template <> struct Arith<__nv_bfloat16> { using type = float; };
 
 // ------------------------------------------------------------------ reductions
-// Sums NQ per-thread partials (double or double-float) over the block (up to
-// 1024 threads) and
-// writes them as doubles to part[bid * NQ + q].  Fixed order:
-// deterministic for a fixed grid.
 // Block index and count a kernel body runs with: the hardware grid for a
 // launch of its own, or one block standing for the whole grid when a
 // persistent kernel runs the body for one instance.
@@ -207,17 +203,47 @@ struct VGrid {
 };
 __device__ __forceinline__ VGrid hw_grid() { return VGrid{(int)blockIdx.x, (int)gridDim.x, (int)blockIdx.x}; }
 
+// Warp sums of N values at once: every exchange halves the values a lane carries (15
+// additions and then 1 for the 14 sums of the step update, where a tree for each takes 70:
+// in FP64, at two lanes a cycle and SM, those were a quarter of a small problem's pass; step
+// update, FP64, n = 1e3, ld = 12: 16.8 -> 12.7 us).  The additions are those of the tree
+// (offsets 16, 8, 4, 2, 1), so the sums have the same bits.  Lane q * (32 / N) ends with
+// value q in v[0].
+__host__ __device__ constexpr int pow2_at_least(int n) { return n <= 1 ? 1 : 2 * pow2_at_least((n + 1) / 2); }
+
+template <int N, int O, typename PA>
+__device__ __forceinline__ void warp_sums_step(PA* v) {
+    if constexpr (O > 0) {
+        if constexpr (N > 1) {
+            const bool up = (threadIdx.x & O) != 0;
+#pragma unroll
+            for (int q = 0; q < N / 2; ++q) {
+                const PA send = up ? v[q] : v[q + N / 2];
+                const PA keep = up ? v[q + N / 2] : v[q];
+                v[q] = keep + shfl_xor(send, O);
+            }
+            warp_sums_step<N / 2, O / 2>(v);
+        } else {
+            v[0] += shfl_xor(v[0], O);
+            warp_sums_step<1, O / 2>(v);
+        }
+    }
+}
+
+// Sums NQ per-thread partials (double or double-float) over the block (up to
+// 1024 threads) and writes them as doubles to part[bid * NQ + q].  Fixed order:
+// deterministic for a fixed grid.
 template <int NQ, typename PA>
 __device__ __forceinline__ void block_partials(PA (&acc)[NQ], double* part, int bid) {
-    __shared__ double red[32][NQ > 0 ? NQ : 1];
+    static_assert(NQ >= 1 && NQ <= 16, "partial sums");
+    __shared__ double red[32][NQ];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    constexpr int P = pow2_at_least(NQ), LV = 32 / P;
+    PA v[P];
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        PA v = acc[q];                       // warp tree in the partial's own type
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += shfl_xor(v, o);
-        if (lane == 0) red[warp][q] = double(v);
-    }
+    for (int q = 0; q < P; ++q) v[q] = q < NQ ? acc[q < NQ ? q : 0] : PA(0);
+    warp_sums_step<P, 16>(v);
+    if (lane % LV == 0 && lane / LV < NQ) red[warp][lane / LV] = double(v[0]);
     __syncthreads();
     for (int q = threadIdx.x; q < NQ; q += blockDim.x) {
         double s = 0.0;
