@@ -104,8 +104,7 @@ k_cons_general(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, cons
             } else {
                 CS yk = CS(0.0), bk;
                 if constexpr (MODE != CONS_ZZ) {
-                    if constexpr (std::is_same_v<CS, double>) yk = y[k];
-                    else yk = ydf ? ld_scalar<CS>(y, ydf, k) : CS(y[k]);
+                    yk = ld_multiplier<CS>(y, ydf, k);
                 }
                 if constexpr (std::is_same_v<CS, double>) bk = __ldg(p.b + k);
                 else bk = p.b_df ? ld_scalar<CS>(p.b, p.b_df, k) : CS(__ldg(p.b + k));
@@ -196,8 +195,7 @@ k_cons_wide(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const T
             if (!act[u]) continue;
             if constexpr (MODE != CONS_EVAL) {
                 if constexpr (MODE != CONS_ZZ) {
-                    if constexpr (std::is_same_v<CS, double>) yk[u] = y[kid[u]];
-                    else yk[u] = ydf ? ld_scalar<CS>(y, ydf, kid[u]) : CS(y[kid[u]]);
+                    yk[u] = ld_multiplier<CS>(y, ydf, kid[u]);
                 }
                 if (MODE == CONS_LS && zk != nullptr) zb[u] = zkc[kid[u]];
                 else if constexpr (std::is_same_v<CS, double>) zb[u] = __ldg(p.b + kid[u]);
@@ -333,6 +331,15 @@ struct LaneDot<dfloat> {
         return r;
     }
 };
+// The same by the type's own multiply-add: the R-only passes over all constraints keep the
+// rounding of their sums (the multiplier step reaches every later iterate).
+template <typename A, typename T1, typename T2>
+__device__ __forceinline__ A dot_exact(const Unit<T1>& x, const Unit<T2>& y) {
+    A s = A(0);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) s = fma(A(x.v[e]), A(y.v[e]), s);
+    return s;
+}
 template <typename A, typename T1, typename T2>
 __device__ __forceinline__ A dot_lane(const Unit<T1>& x, const Unit<T2>& y) {
     LaneDot<A> d;
@@ -442,8 +449,7 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
             }
             if constexpr (MODE != CONS_EVAL) {
                 if constexpr (MODE != CONS_ZZ) {
-                    if constexpr (std::is_same_v<CS, double>) yk = y[kid];
-                    else yk = ydf ? ld_scalar<CS>(y, ydf, kid) : CS(y[kid]);
+                    yk = ld_multiplier<CS>(y, ydf, kid);
                 }
                 if constexpr (MODE == CONS_LS && ZC) zb = zkc[kid];
                 else if constexpr (std::is_same_v<CS, double>) zb = __ldg(p.b + kid);
@@ -493,7 +499,8 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
                         s_1b[u0 + c] = dot_lane<AW>(uj[c][0], vi[c][0]);
                     }
                 } else {
-                    if constexpr (NEED_Z) s_z[u0 + c] = dot_lane<AU>(ui[c][0], uj[c][0]);
+                    if constexpr (MODE == CONS_YTIL) s_z[u0 + c] = dot_lane<AU>(ui[c][0], uj[c][0]);
+                    else if constexpr (NEED_Z) s_z[u0 + c] = dot_exact<AU>(ui[c][0], uj[c][0]);
                     if constexpr (MODE == CONS_LS) {
                         LaneDot<AW> d;
 #pragma unroll

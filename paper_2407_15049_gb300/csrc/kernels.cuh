@@ -243,7 +243,7 @@ k_spmm_c_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld,
                         if constexpr (std::is_same_v<LS, double>) {
                             const double a = __ldg(p.da + i);
                             const double z = zrow ? zrow[i] : a * double(t_rr) - __ldg(p.b + k);
-                            const double yt = __ldg(y + k) - rho * z;
+                            const double yt = ld_multiplier<double>(y, nullptr, k) - rho * z;
                             const double q1 = 2.0 * a * double(t_rd);
                             const double q2 = a * double(t_dd);
                             accq[PL_YQ1] += PA(yt * q1);
@@ -263,7 +263,7 @@ k_spmm_c_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld,
                                                   ld_scalar<dfloat>(p.b, p.b_df, k);
                                 z = LS(zz);
                             }
-                            const LS yv = ydf ? ld_scalar<LS>(y, ydf, k) : LS(__ldg(y + k));
+                            const LS yv = ld_multiplier<LS>(y, ydf, k);
                             const LS yt = yv - rho_s * z;
                             const LS q1 = LS(2) * a * LS(t_rd);
                             const LS q2 = a * LS(t_dd);
@@ -584,7 +584,7 @@ k_update_body(ProbDev p, TR* __restrict__ R, TR* __restrict__ CR, const TDIR* __
                 if (k >= 0) {
                     const RS a = ld_scalar<RS>(p.da, p.da_df, i);
                     const RS z = a * RS(rr) - ld_scalar<RS>(p.b, p.b_df, k);
-                    const RS yv = ydf ? ld_scalar<RS>(y, ydf, k) : RS(__ldg(y + k));
+                    const RS yv = ld_multiplier<RS>(y, ydf, k);
                     coef = AR(a * (yv - rho_r * z));
                     if (rl.lig == 0) {
                         accq[PU_ZZ] += PA(z * z);

@@ -111,6 +111,18 @@ template <> __device__ __forceinline__ float ld_scalar<float>(const double*, con
     return __ldg(reinterpret_cast<const float*>(df + k));     // hi part
 }
 
+// The multiplier y (double, or its double-float mirror): written during a solve, so loaded
+// without the read-only path (the persistent kernels read it after other blocks wrote it).
+template <typename S> __device__ __forceinline__ S ld_multiplier(const double* y, const dfloat* ydf, int64_t k) {
+    if constexpr (std::is_same_v<S, double>) {
+        return y[k];
+    } else {
+        if (ydf == nullptr) return S(y[k]);
+        if constexpr (std::is_same_v<S, dfloat>) return ydf[k];
+        else return ydf[k].hi;
+    }
+}
+
 // type of the per-row z cache (and of the line-search row terms): double on the
 // FP64 path, otherwise the arithmetic type of the direction D
 template <typename TD, typename TR>
