@@ -47,8 +47,9 @@ __device__ __forceinline__ dfloat shfl_xor_in(dfloat v, int o, unsigned m) {
 
 template <typename CS>
 __device__ __forceinline__ CS ld_cs(const double* d, const dfloat* df, int64_t k) {
-    if constexpr (std::is_same_v<CS, double>) return __ldg(d + k);
-    else return df ? ld_scalar<dfloat>(d, df, k) : dfloat(__ldg(d + k));
+    // (the problem's double-float mirrors always exist on a path that is not FP64: a test for
+    // them here would leave the FP64 conversion, predicated off, in every row's instructions)
+    return ld_scalar<CS>(d, df, k);
 }
 
 // ------------------------------------------------------------------ control (one thread)
@@ -124,11 +125,89 @@ __device__ inline void admm_outer_apply(AdmmCtrl* ac, double zz, double by, doub
 //   s = <A_k, X V^T> = a x_i.v_i (i == j) or a (x_i.v_j + x_j.v_i),  z = s - b_k.
 // MODE 0: w_k = y_k - rho z  (written to om, scalar type CS)
 // MODE 1: y_k <- y_k - rho z (and the double-float mirror); partials z^2, b_k y_k.
+// Rows of one unit per lane, one triplet a constraint: groups take constraints in batches
+// with an owner lane each, as k_cons_batch does and for its reasons (with the scalars in one
+// lane of each group the FP64 pipe was 81% busy converting the multipliers).  n = m = 1e6,
+// ld = 20, float rows: 206 -> 56 us.
+template <typename TR, int MODE>
+__device__ __forceinline__ void
+k_admm_cons_batch(ProbDev p, const TR* __restrict__ X, const TR* __restrict__ V, int ld, int L, int Q, double* y,
+                  dfloat* ydf, void* __restrict__ om, const AdmmCtrl* __restrict__ ac, double* __restrict__ part,
+                  VGrid vg) {
+    using AR = arith_t<TR>;
+    using CS = admm_cs_t<TR>;
+    using PA = part_t<TR, TR>;
+    PA accq[PY_N] = {PA(0), PA(0)};
+    const CS rho = CS(ac->rho);
+    constexpr int UC = sizeof(AR) == 8 ? 1 : 2;
+    const int B = L < kConsBatch ? L : kConsBatch;
+    RowLoop rl(L, vg);
+    for (int64_t base = rl.first * B; base < p.m; base += rl.stride * B) {
+        const int64_t t = base + rl.gw * B + rl.lig;
+        const bool own = rl.lig < B && t < p.m;
+        int ii = -1, jj = -1, k = 0;
+        CS a = CS(0.0), bk = CS(0.0), yk = CS(0.0);
+        if (own) {
+            ii = __ldg(p.k_row + t);
+            jj = __ldg(p.k_col + t);
+            k = __ldg(p.k_id + t);
+            a = ld_cs<CS>(p.k_a, p.k_adf, t);
+            bk = ld_cs<CS>(p.b, p.b_df, k);
+            yk = ld_multiplier<CS>(y, ydf, k);
+        }
+        AR s[kConsBatch];
+#pragma unroll
+        for (int u0 = 0; u0 < kConsBatch; u0 += UC) {
+            if (u0 >= B) break;
+            Unit<TR> xi[UC][1], vi[UC][1], xj[UC][1], vj[UC][1];
+            int i[UC], j[UC];
+#pragma unroll
+            for (int c = 0; c < UC; ++c) {
+                i[c] = __shfl_sync(0xffffffffu, ii, rl.base_lane + u0 + c);
+                j[c] = __shfl_sync(0xffffffffu, jj, rl.base_lane + u0 + c);
+                if (u0 + c >= B) i[c] = -1;
+                const int Qa = i[c] >= 0 ? Q : 0;              // no constraint: zero rows
+                const int64_t ri = i[c] >= 0 ? i[c] : 0, rj = i[c] >= 0 ? j[c] : 0;
+                load_row<TR, 1>(xi[c], X, ri, ld, L, Qa, rl.lig);
+                load_row<TR, 1>(vj[c], V, rj, ld, L, Qa, rl.lig);
+                if (i[c] != j[c] && i[c] >= 0) {
+                    load_row<TR, 1>(xj[c], X, rj, ld, L, Q, rl.lig);
+                    load_row<TR, 1>(vi[c], V, ri, ld, L, Q, rl.lig);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < UC; ++c) {
+                s[u0 + c] = dot_lane<AR>(xi[c][0], vj[c][0]);
+                if (i[c] != j[c] && i[c] >= 0) s[u0 + c] = s[u0 + c] + dot_lane<AR>(xj[c][0], vi[c][0]);
+            }
+        }
+        batch_sums(s, L, rl.lig);
+        if (!own) continue;
+        const CS z = a * CS(s[0]) - bk;
+        const CS yn = yk - rho * z;
+        if constexpr (MODE == 0) {
+            static_cast<CS*>(om)[k] = yn;
+        } else {
+            y[k] = double(yn);
+            if (ydf != nullptr) ydf[k] = dfloat(yn);
+            accq[PY_ZZ] += PA(z * z);
+            accq[PY_BY] += PA(bk * yn);
+        }
+    }
+    if constexpr (MODE == 1) block_partials<PY_N>(accq, part, vg.pslot);
+}
+
 template <typename TR, int CPL, int MODE>
 __device__ __forceinline__ void
 k_admm_cons_body(ProbDev p, const TR* __restrict__ X, const TR* __restrict__ V, int ld, int L, int Q,
             double* y, dfloat* ydf, void* __restrict__ om, const AdmmCtrl* __restrict__ ac,
             double* __restrict__ part, VGrid vg) {
+    if constexpr (CPL == 1) {
+        if (p.k_ptr == nullptr) {
+            k_admm_cons_batch<TR, MODE>(p, X, V, ld, L, Q, y, ydf, om, ac, part, vg);
+            return;
+        }
+    }
     using AR = arith_t<TR>;
     using CS = admm_cs_t<TR>;
     using PA = part_t<TR, TR>;
@@ -180,7 +259,8 @@ k_admm_cons_body(ProbDev p, const TR* __restrict__ X, const TR* __restrict__ V, 
             const CS a = p.k_ptr != nullptr ? CS(1.0) : ld_cs<CS>(p.k_a, p.k_adf, t);
             const CS bk = ld_cs<CS>(p.b, p.b_df, k);
             const CS z = a * CS(s) - bk;
-            const CS yk = ld_cs<CS>(y, ydf, k);
+            CS yk;
+            yk = ld_multiplier<CS>(y, ydf, k);
             const CS yn = yk - rho * z;
             if constexpr (MODE == 0) {
                 static_cast<CS*>(om)[k] = yn;
