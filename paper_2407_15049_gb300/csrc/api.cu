@@ -198,7 +198,7 @@ int row_blocks(const lorads_ctx* c, int64_t rows, int L) {
 template <typename TX, typename TO>
 int plan_spmm(const lorads_ctx* c, SpmmCArgs* a) {
     if (a->sh.Q <= 32) {
-        const TilePlan t = tile_plan(c->n, a->sh.Q, c->num_sms * tile_blocks<TX, TO>(), tile_threads<TX, TO>());
+        const TilePlan t = tile_plan(c->n, a->sh.Q, c->num_sms * kTileBlocks, tile_threads<TX, TO>());
         a->nsub = t.nsub;
         a->blocks = t.blocks;
     } else {

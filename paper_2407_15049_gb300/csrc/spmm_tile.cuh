@@ -16,7 +16,7 @@ template <typename TX, typename TO> constexpr int tile_threads() {
     return sizeof(arith_t<TX>) == 8 || sizeof(arith_t<TO>) == 8 ? 128 : 256;
 }
 // Resident blocks the kernel is compiled for.
-template <typename TX, typename TO> constexpr int tile_blocks() { return tile_threads<TX, TO>() == 128 ? 4 : 3; }
+constexpr int kTileBlocks = 4;
 
 // Row groups a warp takes in turn (nsub) and the grid: one resident wave of warps that walk
 // the tiles; small problems take tiles of one row group, so that every row has its lanes.
@@ -56,13 +56,15 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group
 //    is computed, so that a row's gathers wait on no index load;
 //  - the row sums go through shared memory and are taken by lane = row in lane order.
 // Element sums keep the order of the stored entries.  Measured: line search in FP64, n = 1e6,
-// ld = 20, 5e6 entries: 1437 -> 631 us (346 us of FP64 multiply-adds at two lanes a cycle);
-// double-float C R with the objective, n = 1e6, ld = 24: 840 -> 342 us; float product with a
-// multiplier on a 1000 x 1000 torus, ld = 20: 146 -> 121 us.  The line search of the solve keeps
-// k_spmm_c: its scalars are few in float, and the tile form (24 resident warps instead of 32)
-// took 318 us where k_spmm_c takes 224 (n = 1e6, ld = 24).
+// ld = 20, 5e6 entries: 1437 -> 537 us, 631 before the rows were sorted and its sums
+// fused (346 us of FP64 multiply-adds at two lanes a cycle);
+// double-float C R with the objective, n = 1e6, ld = 24: 840 -> 400 us; float product with a
+// multiplier on a 1000 x 1000 torus, ld = 20: 146 -> 121 us with eight gathers in flight a lane and
+// 3 blocks per SM, 89 us with five and 4 (four: 96 us).  The line search of the solve keeps
+// k_spmm_c: its scalars are few in float, and the tile form took 318 us (24 resident warps) where
+// k_spmm_c takes 218 (n = 1e6, ld = 24).
 template <typename TX, typename TO, typename TR, int EPI>
-__global__ void __launch_bounds__((tile_threads<TX, TO>()), (tile_blocks<TX, TO>()))
+__global__ void __launch_bounds__((tile_threads<TX, TO>()), kTileBlocks)
 k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, int Q, int nsub,
             const double* __restrict__ v, int write_out, const TR* __restrict__ R, const double* __restrict__ y,
             double rho_arg, double* __restrict__ part, const Ctrl* gate, int ph) {
@@ -74,8 +76,13 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
     using AW = wide_t<TR, TX>;
     using AD = arith_t<TX>;
     constexpr int NW = tile_threads<TX, TO>() / 32;
-    constexpr int UN = sizeof(AD) == 8 ? 4 : 8;            // gathers in flight per lane
+    constexpr int UN = sizeof(AD) == 8 ? 4 : 5;            // gathers in flight per lane
     constexpr bool kSums = EPI == EPI_LS;
+    // FP64 line search, bound by the FP64 pipe: a row group takes as many steps as the longest of
+    // its rows, so the tile's rows are taken in the order of their lengths, and p1 and p2 are
+    // summed by the multiply-adds themselves
+    constexpr bool kFp64Ls = EPI == EPI_LS && std::is_same_v<A, double>;
+    __shared__ unsigned char s_row[NW][kFp64Ls ? 32 : 1];
     __shared__ __align__(16) int s_col[NW][2][kTileEntries];
     __shared__ __align__(16) TV s_val[NW][2][kTileEntries];
     __shared__ AD s_rd[NW][kSums ? kTileLaneRows : 1], s_dd[NW][kSums ? kTileLaneRows : 1];
@@ -143,21 +150,33 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
         }
         stage_wait<1>();
         __syncwarp();
+        if constexpr (kFp64Ls) {
+            const int mine = own ? my_len : -1;
+            int rank = 0;
+#pragma unroll
+            for (int q = 0; q < 32; ++q) {
+                const int other = __shfl_sync(0xffffffffu, mine, q);
+                rank += other > mine || (other == mine && q < lane) ? 1 : 0;
+            }
+            s_row[wib][rank] = (unsigned char)lane;      // ranks are distinct; lanes without a row come last
+            __syncwarp();
+        }
         const int* sc = s_col[wib][buf];
         const TV* sv = s_val[wib][buf];
         const bool diag = v != nullptr && p.dk != nullptr;
 #pragma unroll 1
         for (int sb = 0; sb < nsub; ++sb) {
-            const int lr = sb * rpw + gw;                  // the group's row of the tile
+            int lr = sb * rpw + gw;                        // the group's row of the tile
+            if constexpr (kFp64Ls) lr = live ? s_row[wib][lr] : 0;
             const int64_t i = r0 + lr;
-            const bool act = live && i < p.n;
+            const bool act = live && lr < rows && i < p.n;
             const int src = live ? lr : 0;
             const int len = __shfl_sync(0xffffffffu, my_len, src);
             // the row's entries: in shared memory, or where they are (generic addresses)
             const int64_t at = __shfl_sync(0xffffffffu, my_at, src);
             const int* rc = in_smem ? sc + (int)at : p.c_col + at;
             const TV* rv = in_smem ? sv + (int)at : cv + at;
-            LaneDot<A> acc[4];
+            A acc[4] = {A(0), A(0), A(0), A(0)};
             Unit<TX> di;
             Unit<TR> ri;
             if (act) {
@@ -185,7 +204,7 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
                 for (int u = 0; u < UN; ++u)
                     if (j[u] >= 0)
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) acc[e].add(A(w[u]), A(x[u].v[e]));
+                        for (int e = 0; e < 4; ++e) acc[e] = fma(A(w[u]), A(x[u].v[e]), acc[e]);
             }
             if (diag) {
                 const int kr = __shfl_sync(0xffffffffu, kc, src);
@@ -195,12 +214,10 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
                     if constexpr (EPI != EPI_NONE) xi = di;
                     else xi.load(X + i * (int64_t)ld + lig * 4);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[e].add(w, A(xi.v[e]));
+                    for (int e = 0; e < 4; ++e) acc[e] = fma(w, A(xi.v[e]), acc[e]);
                 }
             }
-            A o[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) o[e] = acc[e].value();
+            const A(&o)[4] = acc;
             if (write_out && act) {
                 Unit<TO> ou;
 #pragma unroll
@@ -223,17 +240,19 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const AD d = AD(di.v[e]);
-                        p2 = fma(AD(o[e]), d, p2);
+                        if constexpr (kFp64Ls) accq[PL_P2] = fma(AD(o[e]), d, accq[PL_P2]);
+                        else p2 = fma(AD(o[e]), d, p2);
                         rd.add(AD(ri.v[e]), d);
                         dd.add(d, d);
                         const AW r = AW(ri.v[e]);
-                        p1.add(AW(o[e]), r);
+                        if constexpr (kFp64Ls) accq[PL_P1] = fma(AW(o[e]), r, accq[PL_P1]);
+                        else p1.add(AW(o[e]), r);
                         rr.add(r, r);
                     }
-                    accq[PL_P2] += p2;
+                    if constexpr (!kFp64Ls) accq[PL_P2] += p2;
                     s_rd[wib][lr * Q + lig] = rd.value();
                     s_dd[wib][lr * Q + lig] = dd.value();
-                    accq[PL_P1] += PA(AW(2) * p1.value());
+                    if constexpr (!kFp64Ls) accq[PL_P1] += PA(AW(2) * p1.value());
                     s_rr[wib][lr * Q + lig] = rr.value();
                 }
             }
@@ -275,6 +294,7 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
         buf ^= 1;
     }
     stage_wait<0>();
+    if constexpr (kFp64Ls) accq[PL_P1] *= 2.0;
     if constexpr (EPI != EPI_NONE) block_partials<NQ>(accq, part, (int)blockIdx.x);
 }
 
