@@ -11,18 +11,34 @@
 
 namespace lorads {
 
-// ---------------------------------------------------------------- reductions
-// out[q] = sum over blocks of part[b*NQ + q]; warp w folds q = w, w+8, ...
-__device__ void fold_parts(const double* part, int nb, int NQ, double* out) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int q = warp; q < NQ; q += nw) {
-        double s = 0.0;
-        for (int b = lane; b < nb; b += 32) s += part[(size_t)b * NQ + q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) out[q] = s;
+// ---------------------------------------------------------------- control kernels
+// One block, a warp a sum.  What bounds them is the latency of one thread's FP64 code (the
+// root search above all: about 20 us of the root kernel) and, at 1216 blocks, the folds (one
+// SM adds two FP64 numbers a cycle: 8,500 cycles for the step update's 14 sums).  So the sums
+// of all producers are folded at the same time, sixteen loads of a lane in flight, and the
+// control block is worked on in shared memory, where the scalar code's fields are near.  The
+// sums keep their order: a solve's bits are those of the folds one after the other.  History
+// kernel per iteration: n = 1e3, FP64: 14 -> 10.7 us; n = 1e6, mixed: 18 -> 16 us.  (A cluster
+// of eight blocks folding into one: 12.5 and 14 us; its launch costs more than it gives.)
+constexpr int kCtrlThreads = 512;
+
+// out[q] = sum over blocks of part[b*NQ + q]; sums in turn over the block's warps from w0;
+// part null: zeros
+__device__ __forceinline__ void fold_parts(const double* part, int nb, int NQ, double* out, int w0 = 0) {
+    const int nw = blockDim.x >> 5;
+    for (int q = ((int)(threadIdx.x >> 5) - w0 % nw + nw) % nw; q < NQ; q += nw) {
+        const double s = part != nullptr ? fold_one(part, nb, NQ, q) : 0.0;
+        if ((threadIdx.x & 31) == 0) out[q] = s;
     }
 }
+
+// The control block in shared memory: load (before a barrier), store (after one).
+__device__ __forceinline__ void ctrl_load(Ctrl* s, const Ctrl* c) {
+    const int* src = reinterpret_cast<const int*>(c);
+    int* dst = reinterpret_cast<int*>(s);
+    for (int w = threadIdx.x; w < (int)(sizeof(Ctrl) / sizeof(int)); w += blockDim.x) dst[w] = src[w];
+}
+__device__ __forceinline__ void ctrl_store(Ctrl* c, const Ctrl* s) { ctrl_load(c, s); }
 
 __global__ void k_quartic_step(const double* a, double* tau) { *tau = quartic_step(a); }
 
@@ -32,14 +48,16 @@ __global__ void k_quartic_step(const double* a, double* tau) { *tau = quartic_st
 __global__ void k_ctrl_root(Ctrl* c, const double* part_dir, int nb_dir, const double* part_ls, int nb_ls,
                             const double* part_cons, int nb_cons) {
     if (gated_off(c, PH_INNER)) return;
+    __shared__ Ctrl s;
     __shared__ double sd[PD_N], sl[PL_N], sc[PL_N];
+    ctrl_load(&s, c);
     fold_parts(part_dir, nb_dir, PD_N, sd);
-    fold_parts(part_ls, nb_ls, PL_N, sl);
-    if (part_cons != nullptr) fold_parts(part_cons, nb_cons, PL_N, sc);
-    else if (threadIdx.x < PL_N) sc[threadIdx.x] = 0.0;
+    fold_parts(part_ls, nb_ls, PL_N, sl, PD_N);
+    fold_parts(part_cons, nb_cons, PL_N, sc, PD_N + PL_N);
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    ctrl_root_apply(c, sd, sl, sc);
+    if (threadIdx.x == 0) ctrl_root_apply(&s, sd, sl, sc);
+    __syncthreads();
+    ctrl_store(c, &s);
 }
 
 // Standalone variant for lorads_linesearch_coeffs: paper's a4 = p1 - y~^T q1.
@@ -47,8 +65,7 @@ __global__ void k_ls_finish(const double* part_ls, int nb_ls, const double* part
                             double rho, double* out /* a[4], tau */) {
     __shared__ double sl[PL_N], sc[PL_N];
     fold_parts(part_ls, nb_ls, PL_N, sl);
-    if (part_cons != nullptr) fold_parts(part_cons, nb_cons, PL_N, sc);
-    else if (threadIdx.x < PL_N) sc[threadIdx.x] = 0.0;
+    fold_parts(part_cons, nb_cons, PL_N, sc, PL_N);
     __syncthreads();
     if (threadIdx.x != 0) return;
     const double yq1 = sl[PL_YQ1] + sc[PL_YQ1];
@@ -73,15 +90,17 @@ __global__ void k_ctrl_hist(Ctrl* c, int mode, const double* part_upd, int nb_up
     const bool reset = (mode == HIST_RESET);
     if (gated_off(c, reset ? PH_OUTER : PH_INNER)) return;
     const bool fresh = reset || c->step_ok;
+    __shared__ Ctrl s;
     __shared__ double su[PU_N], sy[PC_N];
+    ctrl_load(&s, c);
     if (fresh) {
         fold_parts(part_upd, nb_upd, PU_N, su);
-        if (part_ytil != nullptr) fold_parts(part_ytil, nb_ytil, PC_N, sy);
-        else if (threadIdx.x < PC_N) sy[threadIdx.x] = 0.0;
+        fold_parts(part_ytil, nb_ytil, PC_N, sy, PU_N);
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    ctrl_hist_apply(c, reset, fresh, su, sy);
+    if (threadIdx.x == 0) ctrl_hist_apply(&s, reset, fresh, su, sy);
+    __syncthreads();
+    ctrl_store(c, &s);
 }
 
 // ---------------------------------------------------------------- outer kernel
@@ -93,7 +112,7 @@ __global__ void k_ctrl_outer(Ctrl* c, const double* part_cons, int nb_cons, cons
     if (gated_off(c, PH_OUTER)) return;
     __shared__ double sc[PC_N], so[PO_N];
     fold_parts(part_cons, nb_cons, PC_N, sc);
-    fold_parts(part_obj, nb_obj, PO_N, so);
+    fold_parts(part_obj, nb_obj, PO_N, so, PC_N);
     __syncthreads();
     if (threadIdx.x != 0) return;
     ctrl_outer_apply(c, sc, so);
@@ -103,7 +122,7 @@ __global__ void k_ctrl_outer(Ctrl* c, const double* part_cons, int nb_cons, cons
 __global__ void k_ctrl_init(Ctrl* c, const double* part_cons, int nb_cons, const double* part_obj, int nb_obj) {
     __shared__ double sc[PC_N], so[PO_N];
     fold_parts(part_cons, nb_cons, PC_N, sc);
-    fold_parts(part_obj, nb_obj, PO_N, so);
+    fold_parts(part_obj, nb_obj, PO_N, so, PC_N);
     __syncthreads();
     if (threadIdx.x != 0) return;
     ctrl_init_apply(c, sc, so);
@@ -287,19 +306,19 @@ __global__ void k_lz_tridiag_min(const double* lz, int k, int beta_off, double* 
 
 // ---------------------------------------------------------------- host launchers
 void ctrl_root(cudaStream_t s, Ctrl* c, const double* pd, int nbd, const double* pl, int nbl, const double* pc, int nbc) {
-    k_ctrl_root<<<1, 256, 0, s>>>(c, pd, nbd, pl, nbl, pc, nbc);
+    k_ctrl_root<<<1, kCtrlThreads, 0, s>>>(c, pd, nbd, pl, nbl, pc, nbc);
 }
 void ls_finish(cudaStream_t s, const double* pl, int nbl, const double* pc, int nbc, double rho, double* out) {
-    k_ls_finish<<<1, 256, 0, s>>>(pl, nbl, pc, nbc, rho, out);
+    k_ls_finish<<<1, kCtrlThreads, 0, s>>>(pl, nbl, pc, nbc, rho, out);
 }
 void ctrl_hist(cudaStream_t s, Ctrl* c, int mode, const double* pu, int nbu, const double* py, int nby) {
-    k_ctrl_hist<<<1, 256, 0, s>>>(c, mode, pu, nbu, py, nby);
+    k_ctrl_hist<<<1, kCtrlThreads, 0, s>>>(c, mode, pu, nbu, py, nby);
 }
 void ctrl_outer(cudaStream_t s, Ctrl* c, const double* pc, int nbc, const double* po, int nbo) {
-    k_ctrl_outer<<<1, 256, 0, s>>>(c, pc, nbc, po, nbo);
+    k_ctrl_outer<<<1, kCtrlThreads, 0, s>>>(c, pc, nbc, po, nbo);
 }
 void ctrl_init(cudaStream_t s, Ctrl* c, const double* pc, int nbc, const double* po, int nbo) {
-    k_ctrl_init<<<1, 256, 0, s>>>(c, pc, nbc, po, nbo);
+    k_ctrl_init<<<1, kCtrlThreads, 0, s>>>(c, pc, nbc, po, nbo);
 }
 void ctrl_resume(cudaStream_t s, Ctrl* c) { k_ctrl_resume<<<1, 1, 0, s>>>(c); }
 void quartic_step_dev(cudaStream_t s, const double* a, double* tau) { k_quartic_step<<<1, 1, 0, s>>>(a, tau); }

@@ -32,6 +32,27 @@ __device__ __forceinline__ double normal_at(uint64_t base, int64_t e) {
     return sqrt(-2.0 * log(u1)) * cos(2.0 * 3.141592653589793 * u2);
 }
 
+// ---------------------------------------------------------------- reductions
+// Sum over blocks of part[b*NQ + q] by the calling warp (every lane gets it): lanes stride
+// the blocks, sixteen loads in flight, one addition after the other; then the tree.
+__device__ __forceinline__ double fold_one(const double* __restrict__ part, int nb, int NQ, int q) {
+    constexpr int N = 16;
+    const int lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int b = lane; b < nb; b += 32 * N) {
+        double v[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (b + 32 * k < nb) v[k] = part[(size_t)(b + 32 * k) * NQ + q];
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (b + 32 * k < nb) s += v[k];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 // ---------------------------------------------------------------- cubic root
 __device__ __forceinline__ double qval(const double* a, double t) {
     return ((a[0] * t + a[1]) * t + a[2]) * t * t + a[3] * t;
@@ -170,36 +191,69 @@ __device__ inline void mem_clear(Ctrl* c) {
 // Two-loop recursion of Algorithm 1 (initial matrix I) carried out on
 // coefficients: D = cG G + sum cS_u S_u + sum cY_u Y_u, using only the dot
 // products <G,S_u>, <G,Y_u>, <S_u,Y_v>, <Y_u,Y_v> of the stored pairs.
+// (The pairs' products are read once, in the order of age, into registers: the recursion is
+// a chain of dependent FP64 operations of one thread.)
 __device__ inline void two_loop_coeffs(Ctrl* c) {
     const int mem = c->mem_count;
-    double alpha[kMaxMem];
-    c->cG = -1.0;
-    for (int s = 0; s < kMaxMem; ++s) { c->cS[s] = 0.0; c->cY[s] = 0.0; }
-    for (int t = mem - 1; t >= 0; --t) {                 // newest to oldest
-        const int st = c->order[t];
-        double sD = c->cG * c->g_s[st];
-        for (int u = 0; u < mem; ++u) {
-            const int su = c->order[u];
-            sD += c->cY[su] * c->SY[st][su];
+    double gs[kMaxMem], gy[kMaxMem], SY[kMaxMem][kMaxMem], YY[kMaxMem][kMaxMem];
+    double alpha[kMaxMem], cY[kMaxMem], cS[kMaxMem];
+    int slot[kMaxMem];
+#pragma unroll
+    for (int t = 0; t < kMaxMem; ++t) {
+        slot[t] = c->order[t];
+        cY[t] = cS[t] = alpha[t] = 0.0;
+    }
+#pragma unroll
+    for (int t = 0; t < kMaxMem; ++t) {
+        gs[t] = c->g_s[slot[t]];
+        gy[t] = c->g_y[slot[t]];
+#pragma unroll
+        for (int u = 0; u < kMaxMem; ++u) {
+            SY[t][u] = c->SY[slot[t]][slot[u]];
+            YY[t][u] = c->YY[slot[t]][slot[u]];
         }
-        alpha[t] = sD / c->SY[st][st];
-        c->cY[st] -= alpha[t];
+    }
+    double cG = -1.0;
+#pragma unroll
+    for (int t = kMaxMem - 1; t >= 0; --t) {             // newest to oldest
+        double sD = cG * gs[t];
+#pragma unroll
+        for (int u = 0; u < kMaxMem; ++u)
+            if (u > t && u < mem) sD += cY[u] * SY[t][u];        // cY of the older pairs is still 0
+        if (t < mem) {
+            alpha[t] = sD / SY[t][t];
+            cY[t] -= alpha[t];
+        }
     }
     if (c->lbfgs_scaling && mem > 0) {                   // r = gamma q
-        const int sn = c->order[mem - 1];
-        const double gamma = c->SY[sn][sn] / c->YY[sn][sn];
-        c->cG *= gamma;
-        for (int u = 0; u < mem; ++u) c->cY[c->order[u]] *= gamma;
+        double sy = 0.0, yy = 1.0;
+#pragma unroll
+        for (int t = 0; t < kMaxMem; ++t)
+            if (t == mem - 1) {
+                sy = SY[t][t];
+                yy = YY[t][t];
+            }
+        const double gamma = sy / yy;
+        cG *= gamma;
+#pragma unroll
+        for (int u = 0; u < kMaxMem; ++u) cY[u] *= gamma;
     }
-    for (int t = 0; t < mem; ++t) {                      // oldest to newest
-        const int st = c->order[t];
-        double yD = c->cG * c->g_y[st];
-        for (int u = 0; u < mem; ++u) {
-            const int su = c->order[u];
-            yD += c->cY[su] * c->YY[st][su] + c->cS[su] * c->SY[su][st];
+#pragma unroll
+    for (int t = 0; t < kMaxMem; ++t) {                  // oldest to newest
+        double yD = cG * gy[t];
+#pragma unroll
+        for (int u = 0; u < kMaxMem; ++u)
+            if (u < mem) yD += cY[u] * YY[t][u] + (u < t ? cS[u] * SY[u][t] : 0.0);   // cS of the newer pairs is 0
+        if (t < mem) cS[t] = alpha[t] - yD / SY[t][t];
+    }
+    c->cG = cG;
+    for (int q = 0; q < kMaxMem; ++q) c->cS[q] = c->cY[q] = 0.0;
+#pragma unroll
+    for (int t = 0; t < kMaxMem; ++t)
+        if (t < mem) {
+            c->cS[slot[t]] = cS[t];
+            c->cY[slot[t]] = cY[t];
         }
-        c->cS[st] += alpha[t] - yD / c->SY[st][st];
-    }
 }
 
 // Physical slot of the next pair and the pairs it keeps.
