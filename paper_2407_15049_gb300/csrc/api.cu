@@ -925,6 +925,27 @@ lorads_status run_profiled(lorads_ctx* ctx, int prec, std::chrono::steady_clock:
     return fill_result(ctx, t0, timed_out, res);
 }
 
+// FP64 staging of an n x r factor between the host and the state's type: the history arrays
+// (they hold nothing before the first L-BFGS step and nothing that is read after a solve) when
+// they are large enough, else an allocation of its own.
+struct HostCopy {
+    double* p = nullptr;
+    bool owned = false;
+};
+lorads_status host_copy_begin(lorads_ctx* ctx, HostCopy* h, size_t count) {
+    const SolverState& st = ctx->st;
+    const size_t have = (size_t)ctx->n * st.ld * st.esDir * 2 * (size_t)ctx->prm.lbfgs_mem;
+    if (st.hist && count * sizeof(double) <= have) {
+        h->p = static_cast<double*>(st.hist);
+        return LORADS_OK;
+    }
+    h->owned = true;
+    return dalloc(ctx, &h->p, count);
+}
+void host_copy_end(HostCopy* h) {
+    if (h->owned) dfree(h->p);
+}
+
 // Allocates the solver state for the starting rank and loads R <- R0 (or the
 // device random start) and y <- y0 (or 0), with the double-float mirror of y.
 template <typename TR, typename TD, typename TDIR = TD>
@@ -940,16 +961,28 @@ lorads_status start_state(lorads_ctx* ctx, int prec, const double* R0, int32_t r
     CK(cudaEventRecord(ctx->ev_sync, ctx->stream));
     CK(cudaStreamWaitEvent(ss, ctx->ev_sync, 0));
     const size_t nl = (size_t)ctx->n * st.ld;
-    // R <- R0 (padded to ld, converted to TR)
-    if (R0) {
-        double* tmp = nullptr;
-        if ((s = dalloc(ctx, &tmp, (size_t)ctx->n * r))) return s;
-        CK(cudaMemcpyAsync(tmp, R0, (size_t)ctx->n * r * sizeof(double),
-                           r0_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ss));
-        convert<double, TR>(ss, ctx->n, r, st.ld, r, tmp, st.R, flat_blocks(ctx, (int64_t)nl));
+    // R <- R0 (padded to ld, converted to TR): read where it lies when that is this device, else
+    // copied to the history arrays, which hold nothing yet
+    cudaPointerAttributes at{};
+    bool here = false;
+    if (R0 && r0_on_device) {
+        if (cudaPointerGetAttributes(&at, R0) != cudaSuccess) cudaGetLastError();
+        else here = at.type == cudaMemoryTypeDevice && at.device == ctx->device;
+    }
+    if (here) {
+        convert<double, TR>(ss, ctx->n, r, st.ld, r, R0, st.R, flat_blocks(ctx, (int64_t)nl));
         ctx->launches += 1;
         CK(cudaStreamSynchronize(ss));
-        cudaFree(tmp);
+    } else if (R0) {
+        HostCopy tmp;
+        if ((s = host_copy_begin(ctx, &tmp, (size_t)ctx->n * r))) return s;
+        cudaError_t e = cudaMemcpyAsync(tmp.p, R0, (size_t)ctx->n * r * sizeof(double),
+                                        r0_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ss);
+        if (e == cudaSuccess) convert<double, TR>(ss, ctx->n, r, st.ld, r, tmp.p, st.R, flat_blocks(ctx, (int64_t)nl));
+        ctx->launches += 1;
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ss);
+        host_copy_end(&tmp);
+        CK(e);
     } else {
         CK(cudaMemsetAsync(st.R, 0, nl * sizeof(TR), ss));
         const double scale = std::sqrt(std::max(0.5 * ctx->bnorm1, 1.0) / ((double)ctx->n * r));
@@ -1339,7 +1372,9 @@ lorads_status run_graph(lorads_ctx* ctx, int prec, std::chrono::steady_clock::ti
     SolverState& st = ctx->st;
     cudaStream_t ss = ctx->solve_stream;
     lorads_status s;
-    if ((s = capture<TR, TD, TDIR>(ctx))) return s;
+    // the graph of an earlier solve holds the same kernels and arrays: it is destroyed with the
+    // state's arrays, and nothing else that it was captured from changes
+    if (!st.exec && (s = capture<TR, TD, TDIR>(ctx))) return s;
     constexpr int per_graph = Driver<TR, TD, TDIR>::kInnerPerGraph;
     const int launches = (P.check_every + per_graph - 1) / per_graph;
     // ---- iterate: launch the graph in batches, poll the status of the previous batch
@@ -1552,16 +1587,17 @@ extern "C" lorads_status lorads_get_solution(lorads_ctx* ctx, double* R_host, in
     cudaStream_t s = ctx->solve_stream;
     if (R_host) {
         if (R_capacity < ctx->n * (int64_t)st.r) return set_err(ctx, "R_host too small"), LORADS_ERR_INVALID_ARG;
-        double* tmp = nullptr;
+        HostCopy tmp;
         lorads_status rs;
-        if ((rs = dalloc(ctx, &tmp, (size_t)ctx->n * st.r))) return rs;
+        if ((rs = host_copy_begin(ctx, &tmp, (size_t)ctx->n * st.r))) return rs;
         const int nbk = flat_blocks(ctx, ctx->n * (int64_t)st.r);
-        if (st.rtype == 0) convert<double, double>(s, ctx->n, st.ld, st.r, st.r, st.R, tmp, nbk);
-        else if (st.rtype == 1) convert<dfloat, double>(s, ctx->n, st.ld, st.r, st.r, st.R, tmp, nbk);
-        else convert<float, double>(s, ctx->n, st.ld, st.r, st.r, st.R, tmp, nbk);
-        CK(cudaMemcpyAsync(R_host, tmp, (size_t)ctx->n * st.r * sizeof(double), cudaMemcpyDeviceToHost, s));
-        CK(cudaStreamSynchronize(s));
-        cudaFree(tmp);
+        if (st.rtype == 0) convert<double, double>(s, ctx->n, st.ld, st.r, st.r, st.R, tmp.p, nbk);
+        else if (st.rtype == 1) convert<dfloat, double>(s, ctx->n, st.ld, st.r, st.r, st.R, tmp.p, nbk);
+        else convert<float, double>(s, ctx->n, st.ld, st.r, st.r, st.R, tmp.p, nbk);
+        cudaError_t e = cudaMemcpyAsync(R_host, tmp.p, (size_t)ctx->n * st.r * sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        host_copy_end(&tmp);
+        CK(e);
     }
     if (y_host) {
         CK(cudaMemcpyAsync(y_host, st.y, ctx->m * sizeof(double), cudaMemcpyDeviceToHost, s));
