@@ -714,7 +714,7 @@ struct Driver {
     }
 
     // The captured graph: several L-BFGS iterations, then the outer step's kernels.  Those
-    // return at once where the inner loop goes on, and cost a small problem a fifth of its
+    // return at once where the inner loop goes on, and cost a small problem a tenth of its
     // iteration each time (five launches); an inner loop that ends within the group leaves the
     // rest of it to return at once.  Four: at n = 1e3 an outer step comes every 20 to 50
     // iterations.  Per iteration, n = 1e3, FP64: 86.5 us with one, 78.7 with four (45 us of it the

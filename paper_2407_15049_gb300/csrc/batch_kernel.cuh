@@ -304,7 +304,7 @@ __device__ void batch_solve_one(const BInst& I, const Ctrl& c0, BOut& o, Ctrl* c
                 tick(BP_CONS_LS);
             }
             reduce(SP_DIR, SP_UPD - SP_DIR);          // direction, C pass and constraint pass sums
-            if (tid == 0) ctrl_root_apply(c, tot + SP_DIR, tot + SP_LS, p.m_off ? tot + SP_CLS : tot + SP_ZERO);
+            if (tid < 32) ctrl_root_apply(c, tot + SP_DIR, tot + SP_LS, p.m_off ? tot + SP_CLS : tot + SP_ZERO);
             tm.sync();
             tick(BP_ROOT);
             if (c->solve_done) break;

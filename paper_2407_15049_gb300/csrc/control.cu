@@ -40,7 +40,10 @@ __device__ __forceinline__ void ctrl_load(Ctrl* s, const Ctrl* c) {
 }
 __device__ __forceinline__ void ctrl_store(Ctrl* c, const Ctrl* s) { ctrl_load(c, s); }
 
-__global__ void k_quartic_step(const double* a, double* tau) { *tau = quartic_step(a); }
+__global__ void k_quartic_step(const double* a, double* tau) {
+    const double t = quartic_step(a);
+    if (threadIdx.x == 0) *tau = t;
+}
 
 // ---------------------------------------------------------------- root kernel
 // Folds the line-search partials of the iteration, forms a1..a4 and tau.
@@ -55,7 +58,7 @@ __global__ void k_ctrl_root(Ctrl* c, const double* part_dir, int nb_dir, const d
     fold_parts(part_ls, nb_ls, PL_N, sl, PD_N);
     fold_parts(part_cons, nb_cons, PL_N, sc, PD_N + PL_N);
     __syncthreads();
-    if (threadIdx.x == 0) ctrl_root_apply(&s, sd, sl, sc);
+    if (threadIdx.x < 32) ctrl_root_apply(&s, sd, sl, sc);
     __syncthreads();
     ctrl_store(c, &s);
 }
@@ -67,17 +70,21 @@ __global__ void k_ls_finish(const double* part_ls, int nb_ls, const double* part
     fold_parts(part_ls, nb_ls, PL_N, sl);
     fold_parts(part_cons, nb_cons, PL_N, sc, PL_N);
     __syncthreads();
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x >= 32) return;
     const double yq1 = sl[PL_YQ1] + sc[PL_YQ1];
     const double yq2 = sl[PL_YQ2] + sc[PL_YQ2];
     const double q1q1 = sl[PL_Q1Q1] + sc[PL_Q1Q1];
     const double q1q2 = sl[PL_Q1Q2] + sc[PL_Q1Q2];
     const double q2q2 = sl[PL_Q2Q2] + sc[PL_Q2Q2];
-    out[0] = 0.5 * rho * q2q2;
-    out[1] = rho * q1q2;
-    out[2] = sl[PL_P2] - yq2 + 0.5 * rho * q1q1;
-    out[3] = sl[PL_P1] - yq1;
-    out[4] = quartic_step(out);
+    double a[4];
+    a[0] = 0.5 * rho * q2q2;
+    a[1] = rho * q1q2;
+    a[2] = sl[PL_P2] - yq2 + 0.5 * rho * q1q1;
+    a[3] = sl[PL_P1] - yq1;
+    const double tau = quartic_step(a);
+    if (threadIdx.x != 0) return;
+    for (int q = 0; q < 4; ++q) out[q] = a[q];
+    out[4] = tau;
 }
 
 // ---------------------------------------------------------------- history kernel
@@ -321,7 +328,7 @@ void ctrl_init(cudaStream_t s, Ctrl* c, const double* pc, int nbc, const double*
     k_ctrl_init<<<1, kCtrlThreads, 0, s>>>(c, pc, nbc, po, nbo);
 }
 void ctrl_resume(cudaStream_t s, Ctrl* c) { k_ctrl_resume<<<1, 1, 0, s>>>(c); }
-void quartic_step_dev(cudaStream_t s, const double* a, double* tau) { k_quartic_step<<<1, 1, 0, s>>>(a, tau); }
+void quartic_step_dev(cudaStream_t s, const double* a, double* tau) { k_quartic_step<<<1, 32, 0, s>>>(a, tau); }
 void fold_to(cudaStream_t s, const double* part, int nb, int NQ, double* out) {
     k_fold_to<<<1, 256, 0, s>>>(part, nb, NQ, out);
 }
