@@ -58,7 +58,7 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group
 // Element sums keep the order of the stored entries.  Measured: line search in FP64, n = 1e6,
 // ld = 20, 5e6 entries: 1437 -> 537 us, 631 before the rows were sorted and its sums
 // fused (346 us of FP64 multiply-adds at two lanes a cycle);
-// double-float C R with the objective, n = 1e6, ld = 24: 840 -> 400 us; float product with a
+// double-float C R with the objective, n = 1e6, ld = 24: 840 -> 355 us; float product with a
 // multiplier on a 1000 x 1000 torus, ld = 20: 146 -> 121 us with eight gathers in flight a lane and
 // 3 blocks per SM, 89 us with five and 4 (four: 96 us).  The line search of the solve keeps
 // k_spmm_c: its scalars are few in float, and the tile form took 318 us (24 resident warps) where
