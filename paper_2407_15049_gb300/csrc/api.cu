@@ -768,13 +768,15 @@ lorads_status alloc_state(lorads_ctx* ctx, int prec, int r) {
     if ((s = dalloc(ctx, reinterpret_cast<double**>(&st.zrow), ctx->n))) return s;
     if (!fp64_path && (s = dalloc(ctx, &st.ydf, ctx->m))) return s;
     if ((s = dalloc(ctx, &st.zk, ctx->m))) return s;
-    CK(cudaMemset(st.R, 0, nl * sizeof(TR)));
-    CK(cudaMemset(st.CR, 0, nl * sizeof(TR)));
-    CK(cudaMemset(st.D, 0, nl * sizeof(TDIR)));
-    CK(cudaMemset(st.CD, 0, nl * sizeof(TD)));
-    CK(cudaMemset(st.G, 0, nl * sizeof(TD)));
-    CK(cudaMemset(st.hist, 0, nl * 2 * T * sizeof(TDIR)));
-    if (st.W) CK(cudaMemset(st.W, 0, nl * sizeof(TD)));
+    // cleared on the stream that fills and reads them: it does not wait for the default stream
+    cudaStream_t ss = ctx->solve_stream;
+    CK(cudaMemsetAsync(st.R, 0, nl * sizeof(TR), ss));
+    CK(cudaMemsetAsync(st.CR, 0, nl * sizeof(TR), ss));
+    CK(cudaMemsetAsync(st.D, 0, nl * sizeof(TDIR), ss));
+    CK(cudaMemsetAsync(st.CD, 0, nl * sizeof(TD), ss));
+    CK(cudaMemsetAsync(st.G, 0, nl * sizeof(TD), ss));
+    CK(cudaMemsetAsync(st.hist, 0, nl * 2 * T * sizeof(TDIR), ss));
+    if (st.W) CK(cudaMemsetAsync(st.W, 0, nl * sizeof(TD), ss));
     return LORADS_OK;
 }
 
