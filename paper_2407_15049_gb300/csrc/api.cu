@@ -1019,9 +1019,10 @@ lorads_status admm_ctrl_alloc(lorads_ctx* ctx) {
     return LORADS_OK;
 }
 
-// Work arrays of the stage for row width ld, owned by the context (kept for later calls).
+// Work arrays of the stage for row width ld, owned by the context (kept for later calls), cleared
+// on the stream that uses them.
 template <typename TR, typename TW>
-lorads_status admm_alloc(lorads_ctx* ctx, int ld) {
+lorads_status admm_alloc(lorads_ctx* ctx, int ld, cudaStream_t stream) {
     AdmmState& a = ctx->admm;
     if (a.U && !a.borrowed && a.rtype == type_code<TR>() && a.wtype == type_code<TW>() && a.ld == ld)
         return LORADS_OK;
@@ -1035,9 +1036,9 @@ lorads_status admm_alloc(lorads_ctx* ctx, int ld) {
     if ((s = dalloc(ctx, reinterpret_cast<TW**>(&a.p), nl))) return s;
     if ((s = dalloc(ctx, reinterpret_cast<TW**>(&a.Q), nl))) return s;
     if ((s = dalloc(ctx, reinterpret_cast<double**>(&a.om), ctx->m))) return s;
-    CK(cudaMemset(a.r, 0, nl * sizeof(TW)));
-    CK(cudaMemset(a.p, 0, nl * sizeof(TW)));
-    CK(cudaMemset(a.Q, 0, nl * sizeof(TW)));
+    CK(cudaMemsetAsync(a.r, 0, nl * sizeof(TW), stream));
+    CK(cudaMemsetAsync(a.p, 0, nl * sizeof(TW), stream));
+    CK(cudaMemsetAsync(a.Q, 0, nl * sizeof(TW), stream));
     a.rtype = type_code<TR>();
     a.wtype = type_code<TW>();
     a.ld = ld;
@@ -1061,7 +1062,7 @@ lorads_status admm_bind(lorads_ctx* ctx) {
     const size_t q_bytes = q_in_d ? 0 : nl * sizeof(TW);
     const size_t need = q_bytes + 2 * nl * sizeof(TR);
     const size_t have = nl * st.esDir * 2 * (size_t)ctx->prm.lbfgs_mem;
-    if (need > have || st.esD != sizeof(TW)) return admm_alloc<TR, TW>(ctx, st.ld);
+    if (need > have || st.esD != sizeof(TW)) return admm_alloc<TR, TW>(ctx, st.ld, ctx->solve_stream);
     lorads_status s;
     release_admm_arrays(a);
     if ((s = admm_ctrl_alloc(ctx))) return s;
@@ -1489,7 +1490,7 @@ template <typename TR, typename TW>
 lorads_status run_admm_cg(lorads_ctx* ctx, const void* V, void* X, const double* y, double rho, int ld,
                           const Shape& sh, double cg_rel, int cg_max, int32_t* steps_out) {
     lorads_status s;
-    if ((s = admm_alloc<TR, TW>(ctx, ld))) return s;
+    if ((s = admm_alloc<TR, TW>(ctx, ld, ctx->stream))) return s;
     AdmmState& a = ctx->admm;
     AdmmCtrl h{};
     h.rho = rho;

@@ -28,6 +28,7 @@ def _body(name: str, head: str) -> str:
 
 @pytest.mark.parametrize("name,head", [
     ("api.cu", "lorads_status alloc_state("),
+    ("api.cu", "lorads_status admm_alloc("),
 ])
 def test_clears_name_their_stream(name, head):
     body = _body(name, head)
