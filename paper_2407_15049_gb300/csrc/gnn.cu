@@ -289,10 +289,12 @@ extern "C" lorads_status lorads_gnn_create(lorads_gnn** out, int32_t r_out, int3
     GCREATE(cudaMalloc(&g->m2, pb));
     GCREATE(cudaMalloc(&g->gpart, pb * g->nb));
     GCREATE(cudaMalloc(&g->lpart, sizeof(double) * g->num_sms * 8));
-    GCREATE(cudaMemcpy(g->theta, theta0, pb, cudaMemcpyHostToDevice));
-    GCREATE(cudaMemset(g->m1, 0, pb));
-    GCREATE(cudaMemset(g->m2, 0, pb));
-    GCREATE(cudaMemset(g->grad, 0, pb));
+    // on the caller's stream, which need not wait for the default one
+    GCREATE(cudaMemcpyAsync(g->theta, theta0, pb, cudaMemcpyHostToDevice, g->stream));
+    GCREATE(cudaMemsetAsync(g->m1, 0, pb, g->stream));
+    GCREATE(cudaMemsetAsync(g->m2, 0, pb, g->stream));
+    GCREATE(cudaMemsetAsync(g->grad, 0, pb, g->stream));
+    GCREATE(cudaStreamSynchronize(g->stream));
 #undef GCREATE
     *out = g;
     return LORADS_OK;
@@ -307,10 +309,10 @@ extern "C" lorads_status lorads_gnn_get_params(lorads_gnn* g, float* theta_host,
 
 extern "C" lorads_status lorads_gnn_set_params(lorads_gnn* g, const float* theta_host, int64_t count) {
     if (!g || !theta_host || count < g->P) return LORADS_ERR_INVALID_ARG;
+    GCK(cudaMemcpyAsync(g->theta, theta_host, g->P * sizeof(float), cudaMemcpyHostToDevice, g->stream));
+    GCK(cudaMemsetAsync(g->m1, 0, g->P * sizeof(float), g->stream));
+    GCK(cudaMemsetAsync(g->m2, 0, g->P * sizeof(float), g->stream));
     GCK(cudaStreamSynchronize(g->stream));
-    GCK(cudaMemcpy(g->theta, theta_host, g->P * sizeof(float), cudaMemcpyHostToDevice));
-    GCK(cudaMemset(g->m1, 0, g->P * sizeof(float)));
-    GCK(cudaMemset(g->m2, 0, g->P * sizeof(float)));
     g->step = 0;
     return LORADS_OK;
 }

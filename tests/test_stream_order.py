@@ -29,10 +29,12 @@ def _body(name: str, head: str) -> str:
 @pytest.mark.parametrize("name,head", [
     ("api.cu", "lorads_status alloc_state("),
     ("api.cu", "lorads_status admm_alloc("),
+    ("gnn.cu", 'extern "C" lorads_status lorads_gnn_create('),
+    ("gnn.cu", 'extern "C" lorads_status lorads_gnn_set_params('),
 ])
-def test_clears_name_their_stream(name, head):
+def test_clears_and_copies_name_their_stream(name, head):
     body = _body(name, head)
-    assert not re.search(r"\bcudaMemset\(", body)
+    assert not re.search(r"\bcuda(Memset|Memcpy)\(", body)
 
 
 def _first_iterations(inst, R0, on_device, stream, prec, iters):
