@@ -396,6 +396,9 @@ lorads_status validate_and_build(lorads_ctx* ctx, int64_t n, const int64_t* rp, 
     if ((s = upload(ctx, &ctx->b, b, m))) return s;
     if ((s = upload(ctx, &ctx->k_adf, hp.k_adf.data(), n_trip))) return s;
     if (m_off > 0 && (s = upload(ctx, &ctx->a_adf, hp.a_adf.data(), hp.a_adf.size()))) return s;
+    // The copies run on the default stream and may return before they end; the streams of the
+    // calls that follow need not wait for it.
+    CK(cudaStreamSynchronize(cudaStreamLegacy));
     ProbDev& p = ctx->pd;
     p.n = n; p.m = m;
     p.c_rowptr = ctx->c_rowptr; p.c_col = ctx->c_col; p.c_val = ctx->c_val; p.c_val32 = ctx->c_val32;

@@ -37,6 +37,16 @@ def test_clears_and_copies_name_their_stream(name, head):
     assert not re.search(r"\bcuda(Memset|Memcpy)\(", body)
 
 
+@pytest.mark.parametrize("name,head,last", [
+    ("api.cu", "lorads_status validate_and_build(", "upload("),
+])
+def test_uploads_end_before_the_call_returns(name, head, last):
+    """A copy from pageable memory on the default stream may return before it ends: the call
+    waits for that stream after its last one."""
+    body = _body(name, head)
+    assert body.rfind("cudaStreamSynchronize(cudaStreamLegacy)") > body.rfind(last) > 0
+
+
 def _first_iterations(inst, R0, on_device, stream, prec, iters):
     ctx = L.lorads_create(inst, L.default_params(prec=prec, lbfgs_mem=2), stream=stream.cuda_stream)
     try:
