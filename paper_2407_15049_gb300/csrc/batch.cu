@@ -228,7 +228,8 @@ lorads_status set_iter_limit(lorads_batch* b, int64_t lim) {
     std::vector<Ctrl> h(b->count);
     BCK(cudaMemcpy(h.data(), b->d_ctrl0, sizeof(Ctrl) * b->count, cudaMemcpyDeviceToHost));
     for (auto& c : h) c.total_limit = L;
-    BCK(cudaMemcpy(b->d_ctrl0, h.data(), sizeof(Ctrl) * b->count, cudaMemcpyHostToDevice));
+    BCK(cudaMemcpyAsync(b->d_ctrl0, h.data(), sizeof(Ctrl) * b->count, cudaMemcpyHostToDevice, b->solve_stream));
+    BCK(cudaStreamSynchronize(b->solve_stream));
     return LORADS_OK;
 }
 
@@ -556,6 +557,8 @@ extern "C" lorads_status lorads_batch_create(lorads_batch** out, int32_t count, 
     BCREATE(cudaMalloc(&b->d_order, sizeof(int) * 2 * count));
     BCREATE(cudaMemcpy(b->d_order, ord.data(), sizeof(int) * 2 * count, cudaMemcpyHostToDevice));
     BCREATE(cudaMalloc(&b->d_queue, 2 * sizeof(int)));
+    // the clears and copies above run on the default stream, for which the batch's does not wait
+    BCREATE(cudaStreamSynchronize(cudaStreamLegacy));
     b->shape.ctas_per_sm = std::min(2, max_ctas_per_sm(b->prec, 256));
 #undef BCREATE
     *out = b;

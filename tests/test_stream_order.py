@@ -37,8 +37,14 @@ def test_clears_and_copies_name_their_stream(name, head):
     assert not re.search(r"\bcuda(Memset|Memcpy)\(", body)
 
 
+def test_iteration_limit_of_a_batch_is_set_on_its_stream():
+    body = _body("batch.cu", "lorads_status set_iter_limit(")
+    assert not re.search(r"\bcudaMemcpy\([^;]*HostToDevice", body)
+
+
 @pytest.mark.parametrize("name,head,last", [
     ("api.cu", "lorads_status validate_and_build(", "upload("),
+    ("batch.cu", 'extern "C" lorads_status lorads_batch_create(', "cudaMemcpyHostToDevice"),
 ])
 def test_uploads_end_before_the_call_returns(name, head, last):
     """A copy from pageable memory on the default stream may return before it ends: the call
