@@ -285,16 +285,17 @@ k_spmm_c_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld,
 // off-diagonal constraint pattern:  out = beta_acc * out + alpha * A*_off(v) X
 // VDF: v holds double-float values and each weight alpha a v_k is formed in the
 // output's arithmetic from the double-float coefficient mirror (no FP64
-// operation); otherwise v is double and the weight is formed in FP64.
+// operation); otherwise v is double and the weight is formed in FP64.  v is y~, which a
+// persistent kernel rewrites every iteration: no read-only load.
 template <typename TX, typename TO, int CPL, bool VDF>
 __device__ __forceinline__ A_of_t<TO> spmm_a_weight(const ProbDev& p, const void* v, double alpha, A_of_t<TO> alpha_a,
                                                    int64_t s) {
     using A = A_of_t<TO>;
     const int k = __ldg(p.a_k + s);
     if constexpr (VDF) {
-        return alpha_a * ld_scalar<A>(nullptr, p.a_adf, s) * ld_scalar<A>(nullptr, static_cast<const dfloat*>(v), k);
+        return alpha_a * ld_scalar<A>(nullptr, p.a_adf, s) * ld_multiplier<A>(nullptr, static_cast<const dfloat*>(v), k);
     } else {
-        return A(alpha * __ldg(p.a_a + s) * __ldg(static_cast<const double*>(v) + k));
+        return A(alpha * __ldg(p.a_a + s) * ld_multiplier<double>(static_cast<const double*>(v), nullptr, k));
     }
 }
 

@@ -111,15 +111,19 @@ template <> __device__ __forceinline__ float ld_scalar<float>(const double*, con
     return __ldg(reinterpret_cast<const float*>(df + k));     // hi part
 }
 
-// The multiplier y (double, or its double-float mirror): written during a solve, so loaded
-// without the read-only path (the persistent kernels read it after other blocks wrote it).
+// The multipliers y and y~ (double, or double-float): written during a solve, so loaded without
+// the read-only path (the persistent kernels read them after other blocks wrote them).
 template <typename S> __device__ __forceinline__ S ld_multiplier(const double* y, const dfloat* ydf, int64_t k) {
     if constexpr (std::is_same_v<S, double>) {
         return y[k];
     } else {
         if (ydf == nullptr) return S(y[k]);
-        if constexpr (std::is_same_v<S, dfloat>) return ydf[k];
-        else return ydf[k].hi;
+        if constexpr (std::is_same_v<S, dfloat>) {
+            const float2 v = *reinterpret_cast<const float2*>(ydf + k);
+            return dfloat(v.x, v.y);
+        } else {
+            return ydf[k].hi;
+        }
     }
 }
 
