@@ -478,7 +478,9 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
         }
         // ---- dots of the group's constraints
         AU s_z[kConsBatch];                  // u_i.u_j (R-only modes, EVAL with U == V)
-        AW s_1[kConsBatch], s_1b[kConsBatch];   // EVAL: u_i.v_j and u_j.v_i; LS: their sum in s_1
+        // u_i.v_j and u_j.v_i apart: rounded sums of a float dot each, added in CS (in one float
+        // chain q1 lost a fifth: rms 1.41e-8 -> 1.68e-8 at r = 20)
+        AW s_1[kConsBatch], s_1b[kConsBatch];
         AV s_2[kConsBatch];                  // v_i.v_j
 #pragma unroll
         for (int u0 = 0; u0 < kConsBatch; u0 += UC) {
@@ -522,13 +524,8 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
                     if constexpr (MODE == CONS_YTIL) s_z[u0 + c] = dot_lane<AU>(ui[c][0], uj[c][0]);
                     else if constexpr (NEED_Z) s_z[u0 + c] = dot_exact<AU>(ui[c][0], uj[c][0]);
                     if constexpr (MODE == CONS_LS) {
-                        LaneDot<AW> d;
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            d.add(ui[c][0].v[e], vj[c][0].v[e]);
-                            d.add(uj[c][0].v[e], vi[c][0].v[e]);
-                        }
-                        s_1[u0 + c] = d.value();
+                        s_1[u0 + c] = dot_lane<AW>(ui[c][0], vj[c][0]);
+                        s_1b[u0 + c] = dot_lane<AW>(vi[c][0], uj[c][0]);
                         s_2[u0 + c] = dot_lane<AV>(vi[c][0], vj[c][0]);
                     }
                 }
@@ -545,6 +542,7 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
             if constexpr (NEED_Z) batch_sums(s_z, L, rl.lig);
             if constexpr (MODE == CONS_LS) {
                 batch_sums(s_1, L, rl.lig);
+                batch_sums(s_1b, L, rl.lig);
                 batch_sums(s_2, L, rl.lig);
             }
         }
@@ -565,7 +563,7 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
             else z = fa * CS(s_z[0]) - zb;
             if constexpr (MODE == CONS_LS) {
                 const CS yt = yk - rho_c * z;
-                const CS q1 = fa * CS(s_1[0]);
+                const CS q1 = fa * (CS(s_1[0]) + CS(s_1b[0]));
                 const CS q2 = fa * CS(s_2[0]);
                 accq[PL_YQ1] += PA(yt * q1);
                 accq[PL_YQ2] += PA(yt * q2);
