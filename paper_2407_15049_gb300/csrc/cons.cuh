@@ -294,58 +294,13 @@ k_cons_wide(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const T
     if constexpr (MODE != CONS_EVAL) block_partials<NQ>(accq, part, vg.pslot);
 }
 
-// Per-lane partial dot of gathered rows.  Float and double: a chain of fused
-// multiply-adds.  Double-float: exact products (two_prod, and the cross terms in one
-// float) added by TwoSum, the errors collected in a float of their own; about 12
-// operations an element instead of the 30 of a double-word multiply and add, with the
-// same error term (each error sum is rounded at 2^-24 of a quantity 2^-24 of the dot).
-template <typename A>
-struct LaneDot {
-    A s = A(0);
-    template <typename T1, typename T2>
-    __device__ __forceinline__ void add(T1 x, T2 y) { s = fma(A(x), A(y), s); }
-    __device__ __forceinline__ A value() const { return s; }
-};
-template <>
-struct LaneDot<dfloat> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void take(float p, float e) {
-        float t;
-        two_sum(hi, p, hi, t);
-        lo = __fadd_rn(lo, __fadd_rn(t, e));
-    }
-    __device__ __forceinline__ void add(dfloat x, dfloat y) {
-        float p, e;
-        two_prod(x.hi, y.hi, p, e);
-        take(p, __fmaf_rn(x.lo, y.hi, __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.lo, e))));
-    }
-    __device__ __forceinline__ void add(dfloat x, float y) {
-        float p, e;
-        two_prod(x.hi, y, p, e);
-        take(p, __fmaf_rn(x.lo, y, e));
-    }
-    __device__ __forceinline__ void add(float x, dfloat y) { add(y, x); }
-    __device__ __forceinline__ dfloat value() const {
-        dfloat r;
-        two_sum(hi, lo, r.hi, r.lo);
-        return r;
-    }
-};
-// The same by the type's own multiply-add: the R-only passes over all constraints keep the
-// rounding of their sums (the multiplier step reaches every later iterate).
+// Per-lane partial dot of gathered rows, by the arithmetic type's own multiply-add.
 template <typename A, typename T1, typename T2>
-__device__ __forceinline__ A dot_exact(const Unit<T1>& x, const Unit<T2>& y) {
+__device__ __forceinline__ A dot_lane(const Unit<T1>& x, const Unit<T2>& y) {
     A s = A(0);
 #pragma unroll
     for (int e = 0; e < 4; ++e) s = fma(A(x.v[e]), A(y.v[e]), s);
     return s;
-}
-template <typename A, typename T1, typename T2>
-__device__ __forceinline__ A dot_lane(const Unit<T1>& x, const Unit<T2>& y) {
-    LaneDot<A> d;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) d.add(x.v[e], y.v[e]);
-    return d.value();
 }
 
 // Sums of up to kConsBatch values over the L lanes of a group at once: v[u] of every
@@ -521,8 +476,7 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
                         s_1b[u0 + c] = dot_lane<AW>(uj[c][0], vi[c][0]);
                     }
                 } else {
-                    if constexpr (MODE == CONS_YTIL) s_z[u0 + c] = dot_lane<AU>(ui[c][0], uj[c][0]);
-                    else if constexpr (NEED_Z) s_z[u0 + c] = dot_exact<AU>(ui[c][0], uj[c][0]);
+                    if constexpr (NEED_Z) s_z[u0 + c] = dot_lane<AU>(ui[c][0], uj[c][0]);
                     if constexpr (MODE == CONS_LS) {
                         s_1[u0 + c] = dot_lane<AW>(ui[c][0], vj[c][0]);
                         s_1b[u0 + c] = dot_lane<AW>(vi[c][0], uj[c][0]);

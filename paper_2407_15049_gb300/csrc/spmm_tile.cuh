@@ -226,34 +226,33 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
             }
             if constexpr (EPI == EPI_OBJ) {
                 if (act) {
-                    LaneDot<A> d;
+                    A d = A(0);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) d.add(o[e], A(di.v[e]));
-                    accq[PO_CRR] += PA(d.value());
+                    for (int e = 0; e < 4; ++e) d = fma(o[e], A(di.v[e]), d);
+                    accq[PO_CRR] += PA(d);
                 }
             }
             if constexpr (EPI == EPI_LS) {
                 if (act) {
-                    AD p2 = AD(0);
-                    LaneDot<AD> rd, dd;
-                    LaneDot<AW> p1, rr;
+                    AD p2 = AD(0), rd = AD(0), dd = AD(0);
+                    AW p1 = AW(0), rr = AW(0);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const AD d = AD(di.v[e]);
                         if constexpr (kFp64Ls) accq[PL_P2] = fma(AD(o[e]), d, accq[PL_P2]);
                         else p2 = fma(AD(o[e]), d, p2);
-                        rd.add(AD(ri.v[e]), d);
-                        dd.add(d, d);
+                        rd = fma(AD(ri.v[e]), d, rd);
+                        dd = fma(d, d, dd);
                         const AW r = AW(ri.v[e]);
                         if constexpr (kFp64Ls) accq[PL_P1] = fma(AW(o[e]), r, accq[PL_P1]);
-                        else p1.add(AW(o[e]), r);
-                        rr.add(r, r);
+                        else p1 = fma(AW(o[e]), r, p1);
+                        rr = fma(r, r, rr);
                     }
                     if constexpr (!kFp64Ls) accq[PL_P2] += p2;
-                    s_rd[wib][lr * Q + lig] = rd.value();
-                    s_dd[wib][lr * Q + lig] = dd.value();
-                    if constexpr (!kFp64Ls) accq[PL_P1] += PA(AW(2) * p1.value());
-                    s_rr[wib][lr * Q + lig] = rr.value();
+                    s_rd[wib][lr * Q + lig] = rd;
+                    s_dd[wib][lr * Q + lig] = dd;
+                    if constexpr (!kFp64Ls) accq[PL_P1] += PA(AW(2) * p1);
+                    s_rr[wib][lr * Q + lig] = rr;
                 }
             }
         }

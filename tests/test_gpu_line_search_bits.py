@@ -3,6 +3,9 @@
 Each input is chosen so that the value is exact in the arithmetic that the pass states, and
 not in a cheaper one, so the expected value is exact and has no tolerance.
 """
+import math
+from fractions import Fraction
+
 import numpy as np
 import pytest
 import torch
@@ -42,3 +45,62 @@ def test_q1_adds_its_two_dots_beyond_float(ld, dtype, swap):
         L.lorads_destroy(ctx)
     assert a[3] == -2.0 * (2.0**24 + 1.0)
     assert a[0] == a[1] == a[2] == 0.0
+
+
+def _f32(q: Fraction) -> Fraction:
+    """q rounded to the nearest float (ties to even; the values here are normal)."""
+    if q == 0:
+        return q
+    e = math.floor(math.log2(abs(q)))
+    while abs(q) >= Fraction(2) ** (e + 1):
+        e += 1
+    while abs(q) < Fraction(2) ** e:
+        e -= 1
+    ulp = Fraction(2) ** (e - 23)
+    return Fraction(round(q / ulp)) * ulp
+
+
+def _two_sum(a, b):
+    s = _f32(a + b)
+    return s, a + b - s
+
+
+def _dw_mul(x, y):
+    """DWTimesDW with fused multiply-adds (Joldes, Muller, Popescu 2017)."""
+    ch = _f32(x[0] * y[0])
+    cl1 = x[0] * y[0] - ch
+    cl2 = _f32(x[1] * y[0] + _f32(x[0] * y[1] + _f32(x[1] * y[1])))
+    return _two_sum(ch, _f32(cl1 + cl2))
+
+
+def _dw_add(x, y):
+    """AccurateDWPlusDW of the same paper."""
+    sh, sl = _two_sum(x[0], y[0])
+    th, tl = _two_sum(x[1], y[1])
+    vh, vl = _two_sum(sh, _f32(sl + th))
+    return _two_sum(vh, _f32(tl + vl))
+
+
+def test_double_float_dots_are_double_word_multiply_adds():
+    """The objective at the start of a double-float solve, for a C of one stored diagonal entry 1 and rows
+    of four elements: one lane's dot, the double-word multiply-add of its elements in turn."""
+    n = 5
+    rowptr = np.zeros(n + 1, dtype=np.int64)
+    rowptr[3:] = 1
+    inst = W.SDPInstance(n=n, rowptr=rowptr, colind=np.array([2], np.int32), val=np.array([1.0]), m=n,
+                         con=np.arange(n, dtype=np.int32), row=np.arange(n, dtype=np.int32),
+                         col=np.arange(n, dtype=np.int32), aval=np.ones(n), b=np.ones(n), kind="generic")
+    ctx = L.lorads_create(inst, L.default_params(prec=L.LORADS_DF64, max_outer=1, tol=1e-300))
+    rng = np.random.default_rng(11)
+    try:
+        for _ in range(40):
+            R0 = rng.standard_normal((n, 4))
+            got = L.lorads_solve(ctx, R0, max_total_inner=1)["primal_obj"]
+            acc = (Fraction(0), Fraction(0))
+            for v in R0[2]:
+                hi = Fraction(float(np.float32(v)))
+                x = (hi, _f32(Fraction(float(v)) - hi))
+                acc = _dw_add(_dw_mul(x, x), acc)
+            assert got == float(acc[0] + acc[1])
+    finally:
+        L.lorads_destroy(ctx)
