@@ -54,7 +54,7 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group
 //    and the line-search scalars formed by lane = row, once per tile;
 //  - the stored entries of the next tile are copied to shared memory (cp.async) while this one
 //    is computed, so that a row's gathers wait on no index load;
-//  - the row sums go through shared memory and are taken by lane = row in lane order.
+//  - the row sums go through shared memory and are taken by lane = row.
 // Element sums keep the order of the stored entries.  Measured: line search in FP64, n = 1e6,
 // ld = 20, 5e6 entries: 1437 -> 537 us, 631 before the rows were sorted and its sums
 // fused (346 us of FP64 multiply-adds at two lanes a cycle);
@@ -259,13 +259,17 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
         __syncwarp();
         if constexpr (EPI == EPI_LS) {
             if (kc >= 0) {
-                AD t_rd = s_rd[wib][lane * Q], t_dd = s_dd[wib][lane * Q];
-                AW t_rr = s_rr[wib][lane * Q];
-                for (int q = 1; q < Q; ++q) {
-                    t_rd += s_rd[wib][lane * Q + q];
-                    t_dd += s_dd[wib][lane * Q + q];
-                    t_rr += s_rr[wib][lane * Q + q];
-                }
+                // the tree of group_sum over the row's lanes (a chain of up to 32 would round more)
+                AD *rd = s_rd[wib] + lane * Q, *dd = s_dd[wib] + lane * Q;
+                AW* rr = s_rr[wib] + lane * Q;
+                for (int h = Q > 1 ? 1 << (31 - __clz(Q - 1)) : 0; h > 0; h >>= 1)
+                    for (int q = 0; q < h && q + h < Q; ++q) {
+                        rd[q] += rd[q + h];
+                        dd[q] += dd[q + h];
+                        rr[q] += rr[q + h];
+                    }
+                const AD t_rd = rd[0], t_dd = dd[0];
+                const AW t_rr = rr[0];
                 LS a, z, yv;
                 if constexpr (std::is_same_v<LS, double>) {
                     a = __ldg(p.da + my);

@@ -47,6 +47,29 @@ def test_q1_adds_its_two_dots_beyond_float(ld, dtype, swap):
     assert a[0] == a[1] == a[2] == 0.0
 
 
+@pytest.mark.parametrize("ld", [16, 20, 24, 32, 64, 128, 256])
+@pytest.mark.parametrize("dtype,big", [(torch.float32, 4096.0), (torch.bfloat16, 4096.0), (torch.float64, 2.0**27)])
+def test_row_sums_add_as_a_tree(ld, dtype, big):
+    """r_i.d_i of a diagonal constraint, with big^2, 1, -big^2 in the first, second and (L/2)-th group of
+    four elements, L the lanes of a row: the tree over the lanes pairs the first with the third and
+    keeps the 1, a chain over them loses it."""
+    n, i = 9, 4
+    lanes = 1
+    while lanes < min(ld // 4, 32):
+        lanes *= 2
+    inst = _one_offdiagonal(n, i, i)
+    R = torch.zeros((n, ld), dtype=dtype, device="cuda")
+    D = torch.zeros((n, ld), dtype=dtype, device="cuda")
+    for unit, r, d in ((0, big, big), (1, 1.0, 1.0), (lanes // 2, big, -big)):
+        R[i, 4 * unit], D[i, 4 * unit] = r, d
+    ctx = L.lorads_create(inst)
+    try:
+        a, _ = L.lorads_linesearch_coeffs(ctx, R, D, torch.full((1,), 1.0, dtype=torch.float64, device="cuda"), 0.0)
+    finally:
+        L.lorads_destroy(ctx)
+    assert a[3] == -2.0
+
+
 def _f32(q: Fraction) -> Fraction:
     """q rounded to the nearest float (ties to even; the values here are normal)."""
     if q == 0:
