@@ -79,8 +79,9 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
     constexpr int UN = sizeof(AD) == 8 ? 4 : 5;            // gathers in flight per lane
     constexpr bool kSums = EPI == EPI_LS;
     // FP64 line search, bound by the FP64 pipe: a row group takes as many steps as the longest of
-    // its rows, so the tile's rows are taken in the order of their lengths, and p1 and p2 are
-    // summed by the multiply-adds themselves
+    // its rows, so the tile's rows are taken in the order of their lengths, and a tile's p1 and p2
+    // are summed by the multiply-adds themselves (through one sum for the whole walk, four times the
+    // additions to it, the coefficients' error grew from 1.6e-17 to 1.4e-16)
     constexpr bool kFp64Ls = EPI == EPI_LS && std::is_same_v<A, double>;
     __shared__ unsigned char s_row[NW][kFp64Ls ? 32 : 1];
     __shared__ __align__(16) int s_col[NW][2][kTileEntries];
@@ -164,6 +165,7 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
         const int* sc = s_col[wib][buf];
         const TV* sv = s_val[wib][buf];
         const bool diag = v != nullptr && p.dk != nullptr;
+        double t_p1 = 0.0, t_p2 = 0.0;                     // the tile's, in the FP64 line search
 #pragma unroll 1
         for (int sb = 0; sb < nsub; ++sb) {
             int lr = sb * rpw + gw;                        // the group's row of the tile
@@ -239,12 +241,12 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const AD d = AD(di.v[e]);
-                        if constexpr (kFp64Ls) accq[PL_P2] = fma(AD(o[e]), d, accq[PL_P2]);
+                        if constexpr (kFp64Ls) t_p2 = fma(AD(o[e]), d, t_p2);
                         else p2 = fma(AD(o[e]), d, p2);
                         rd = fma(AD(ri.v[e]), d, rd);
                         dd = fma(d, d, dd);
                         const AW r = AW(ri.v[e]);
-                        if constexpr (kFp64Ls) accq[PL_P1] = fma(AW(o[e]), r, accq[PL_P1]);
+                        if constexpr (kFp64Ls) t_p1 = fma(AW(o[e]), r, t_p1);
                         else p1 = fma(AW(o[e]), r, p1);
                         rr = fma(r, r, rr);
                     }
@@ -257,6 +259,10 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
             }
         }
         __syncwarp();
+        if constexpr (kFp64Ls) {
+            accq[PL_P1] += 2.0 * t_p1;
+            accq[PL_P2] += t_p2;
+        }
         if constexpr (EPI == EPI_LS) {
             if (kc >= 0) {
                 // the tree of group_sum over the row's lanes (a chain of up to 32 would round more)
@@ -297,7 +303,6 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
         buf ^= 1;
     }
     stage_wait<0>();
-    if constexpr (kFp64Ls) accq[PL_P1] *= 2.0;
     if constexpr (EPI != EPI_NONE) block_partials<NQ>(accq, part, (int)blockIdx.x);
 }
 

@@ -70,6 +70,30 @@ def test_row_sums_add_as_a_tree(ld, dtype, big):
     assert a[3] == -2.0
 
 
+def test_fp64_line_search_sums_its_rows_before_the_walk():
+    """C = I and every four elements of R = D with the squares e, e, e, 1, e = 2^-48.  A thread walks 128
+    rows, so its sum grows to 128 and e is half an ulp of it or less from 32 on: added one by one
+    they are lost (8e-15 of the sum).  Added a tile at a time the sum takes at most 128 additions of
+    at least one row, 22 for tiles of six, each off by half an ulp of 128 at most: 1.2e-15, and the
+    folds over the blocks round a dozen times (1.3e-15)."""
+    ld, e = 128, 2.0**-48
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * 4 * 4
+    n = 128 * warps
+    inst = W.SDPInstance(n=n, rowptr=np.arange(n + 1, dtype=np.int64), colind=np.arange(n, dtype=np.int32),
+                         val=np.ones(n), m=1, con=np.array([0], np.int32), row=np.array([0], np.int32),
+                         col=np.array([0], np.int32), aval=np.array([1.0]), b=np.array([1.0]), kind="generic")
+    row = torch.tensor([2.0**-24] * 3 + [1.0], dtype=torch.float64, device="cuda").repeat(ld // 4)
+    R = row.repeat(n, 1).contiguous()
+    ctx = L.lorads_create(inst)
+    try:
+        a, _ = L.lorads_linesearch_coeffs(ctx, R, R.clone(), torch.zeros(1, dtype=torch.float64, device="cuda"), 0.0)
+    finally:
+        L.lorads_destroy(ctx)
+    want = n * (ld // 4) * (1 + 3 * Fraction(e))
+    assert abs(Fraction(float(a[2])) - want) <= Fraction(2.5e-15) * want
+    assert abs(Fraction(float(a[3])) - 2 * want) <= Fraction(2.5e-15) * 2 * want
+
+
 def _f32(q: Fraction) -> Fraction:
     """q rounded to the nearest float (ties to even; the values here are normal)."""
     if q == 0:
