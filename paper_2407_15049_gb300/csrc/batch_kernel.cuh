@@ -213,13 +213,18 @@ __device__ void batch_solve_one(const BInst& I, const Ctrl& c0, BOut& o, Ctrl* c
         k_spmm_c_body<TR, TR, TR, 1, EPI_OBJ>(p, R, CR, ld, L, Q, nullptr, 1, R, y, nullptr, nullptr, c, 0.0,
                                                sp + SP_OBJ, vg);
     };
+    // W = A*_off(y~) R
+    auto pattern_product = [&]() {
+        if (L <= 2) k_spmm_a_body<TR, TD, 1, kYtilDf, true>(p, R, W, ld, L, Q, ytil, 1.0, 0, vg);
+        else k_spmm_a_body<TR, TD, 1, kYtilDf, false>(p, R, W, ld, L, Q, ytil, 1.0, 0, vg);
+    };
     // G = grad L at the current R, then a fresh inner loop (memory empty)
     auto outer_gradient = [&]() {
         if (p.m_off) {
             k_cons_body<TR, TR, 1, CONS_YTIL>(p, p.m_diag, p.m, R, R, ld, L, Q, y, ytil, zk, ydf, c, 0.0,
                                               sp + SP_YT, vg);
             tm.sync();
-            k_spmm_a_body<TR, TD, 1, kYtilDf>(p, R, W, ld, L, Q, ytil, 1.0, 0, vg);
+            pattern_product();
             tm.sync();
         }
         k_update_body<TR, TD, 1, false, false>(p, R, CR, D, CD, G, p.m_off ? W : nullptr, hist, sstride, ld, L, Q,
@@ -317,7 +322,7 @@ __device__ void batch_solve_one(const BInst& I, const Ctrl& c0, BOut& o, Ctrl* c
                                                       sp + SP_YT, vg);
                     tm.sync();
                     tick(BP_YTIL);
-                    k_spmm_a_body<TR, TD, 1, kYtilDf>(p, R, W, ld, L, Q, ytil, 1.0, 0, vg);
+                    pattern_product();
                     tm.sync();
                     tick(BP_SPMM_A);
                     k_update_body<TR, TD, 1, false, true>(p, R, CR, D, CD, G, W, hist, sstride, ld, L, Q, y, ydf,

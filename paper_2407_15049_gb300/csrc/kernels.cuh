@@ -299,7 +299,47 @@ __device__ __forceinline__ A_of_t<TO> spmm_a_weight(const ProbDev& p, const void
     }
 }
 
+// acc += the weighted rows of the slots [s, s1), four slots in flight, each weight formed by
+// every lane.  For groups of one and two lanes, which have little to share.
 template <typename TX, typename TO, int CPL, bool VDF>
+__device__ __forceinline__ void
+spmm_a_row_narrow(const ProbDev& p, const TX* __restrict__ X, int ld, int L, int Q, const void* __restrict__ v,
+                  double alpha, int lig, int64_t s, int64_t s1, A_of_t<TO> (&acc)[CPL][4]) {
+    using A = A_of_t<TO>;
+    const A alpha_a = A(alpha);
+    constexpr int UN = 4;
+    for (; s + UN <= s1; s += UN) {
+        int j[UN];
+        A w[UN];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) {
+            j[u] = __ldg(p.a_col + s + u);
+            w[u] = spmm_a_weight<TX, TO, CPL, VDF>(p, v, alpha, alpha_a, s + u);
+        }
+        Unit<TX> x[UN][CPL];
+#pragma unroll
+        for (int u = 0; u < UN; ++u) load_row<TX, CPL>(x[u], X, j[u], ld, L, Q, lig);
+#pragma unroll
+        for (int u = 0; u < UN; ++u)
+#pragma unroll
+            for (int c = 0; c < CPL; ++c)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[c][e] = fma(w[u], A(x[u][c].v[e]), acc[c][e]);
+    }
+    for (; s < s1; ++s) {
+        const int j = __ldg(p.a_col + s);
+        const A w = spmm_a_weight<TX, TO, CPL, VDF>(p, v, alpha, alpha_a, s);
+        Unit<TX> x[CPL];
+        load_row<TX, CPL>(x, X, j, ld, L, Q, lig);
+#pragma unroll
+        for (int c = 0; c < CPL; ++c)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[c][e] = fma(w, A(x[c].v[e]), acc[c][e]);
+    }
+}
+
+// NARROW: groups of one or two lanes (L <= 2), else L >= 4.
+template <typename TX, typename TO, int CPL, bool VDF, bool NARROW>
 __device__ __forceinline__ void
 k_spmm_a_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, int L, int Q,
          const void* __restrict__ v, double alpha, int accumulate, VGrid vg) {
@@ -309,10 +349,11 @@ k_spmm_a_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld,
     // Slots per trip of a group: lane u loads slot u of the batch (coalesced) and forms
     // its weight; the rows are then gathered with the slots broadcast by shuffles.  Forming
     // each weight in every lane of the group made the pass FP64-bound where v is double (two
-    // products and a conversion per slot and lane).  Measured: 5.4e6 slots on 1e5 rows of 24
-    // bf16 elements, v double: 308 -> 170 us; 2e6 slots, double-float rows and v: 66 -> 54 us.
+    // products and a conversion per slot and lane).
     const int B = L < 8 ? L : 8;
     constexpr int UN = CPL == 1 ? (sizeof(TX) == 8 ? 4 : 8) : 2;     // rows in flight per lane
+    // bf16 rows: a slot past the end loads a row of zeros under a mask in place of a branch
+    constexpr bool kMasked = sizeof(TX) == 2;
     for (int64_t base = rl.first; base < p.n; base += rl.stride) {
         const int64_t i = base + rl.gw;
         const bool act = i < p.n;
@@ -322,38 +363,46 @@ k_spmm_a_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld,
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[c][e] = A(0);
         const int64_t s0 = act ? __ldg(p.a_rowptr + i) : 0, s1 = act ? __ldg(p.a_rowptr + i + 1) : 0;
-        // warp-uniform loop: the groups of a warp may hold different numbers of slots
-        for (int64_t s = s0; __any_sync(0xffffffffu, s < s1); s += B) {
-            const int64_t q = s + rl.lig;
-            int jo = -1;
-            A wo = A(0);
-            if (rl.lig < B && q < s1) {
-                jo = __ldg(p.a_col + q);
-                wo = spmm_a_weight<TX, TO, CPL, VDF>(p, v, alpha, alpha_a, q);
-            }
-#pragma unroll
-            for (int u0 = 0; u0 < 8; u0 += UN) {
-                if (u0 >= B) break;
-                int j[UN];
-                A w[UN];
-                Unit<TX> x[UN][CPL];
-#pragma unroll
-                for (int u = 0; u < UN; ++u) {
-                    const int src = rl.base_lane + (u0 + u < B ? u0 + u : 0);
-                    j[u] = __shfl_sync(0xffffffffu, jo, src);
-                    w[u] = shfl_idx(wo, src);
-                    if (u0 + u >= B) j[u] = -1;
+        if constexpr (NARROW) {
+            spmm_a_row_narrow<TX, TO, CPL, VDF>(p, X, ld, L, Q, v, alpha, rl.lig, s0, s1, acc);
+        } else {
+            // warp-uniform loop: the groups of a warp may hold different numbers of slots
+            for (int64_t s = s0; __any_sync(0xffffffffu, s < s1); s += B) {
+                const int64_t q = s + rl.lig;
+                int jo = -1;
+                A wo = A(0);
+                if (rl.lig < B && q < s1) {
+                    jo = __ldg(p.a_col + q);
+                    wo = spmm_a_weight<TX, TO, CPL, VDF>(p, v, alpha, alpha_a, q);
                 }
 #pragma unroll
-                for (int u = 0; u < UN; ++u)
-                    if (j[u] >= 0) load_row<TX, CPL>(x[u], X, j[u], ld, L, Q, rl.lig);
+                for (int u0 = 0; u0 < 8; u0 += UN) {
+                    if (u0 >= B) break;
+                    int j[UN];
+                    A w[UN];
+                    Unit<TX> x[UN][CPL];
 #pragma unroll
-                for (int u = 0; u < UN; ++u)
-                    if (j[u] >= 0)
+                    for (int u = 0; u < UN; ++u) {
+                        const int src = rl.base_lane + (u0 + u < B ? u0 + u : 0);
+                        j[u] = __shfl_sync(0xffffffffu, jo, src);
+                        w[u] = shfl_idx(wo, src);
+                        if (u0 + u >= B) j[u] = -1;
+                    }
 #pragma unroll
-                        for (int c = 0; c < CPL; ++c)
+                    for (int u = 0; u < UN; ++u) {
+                        if constexpr (kMasked)
+                            load_row<TX, CPL>(x[u], X, j[u] >= 0 ? j[u] : 0, ld, L, j[u] >= 0 ? Q : 0, rl.lig);
+                        else if (j[u] >= 0)
+                            load_row<TX, CPL>(x[u], X, j[u], ld, L, Q, rl.lig);
+                    }
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) acc[c][e] = fma(w[u], A(x[u][c].v[e]), acc[c][e]);
+                    for (int u = 0; u < UN; ++u)
+                        if (j[u] >= 0)
+#pragma unroll
+                            for (int c = 0; c < CPL; ++c)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) acc[c][e] = fma(w[u], A(x[u][c].v[e]), acc[c][e]);
+                }
             }
         }
         if (!act) continue;
@@ -684,12 +733,12 @@ k_spmm_c(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, int 
                                                    part, hw_grid());
 }
 
-template <typename TX, typename TO, int CPL, bool VDF>
+template <typename TX, typename TO, int CPL, bool VDF, bool NARROW>
 __global__ void __launch_bounds__(kThreads)
 k_spmm_a(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, int L, int Q,
          const void* __restrict__ v, double alpha, int accumulate, const Ctrl* gate, int ph) {
     if (gated_off(gate, ph)) return;
-    k_spmm_a_body<TX, TO, CPL, VDF>(p, X, out, ld, L, Q, v, alpha, accumulate, hw_grid());
+    k_spmm_a_body<TX, TO, CPL, VDF, NARROW>(p, X, out, ld, L, Q, v, alpha, accumulate, hw_grid());
 }
 
 template <typename TU, typename TV, int CPL, int MODE>

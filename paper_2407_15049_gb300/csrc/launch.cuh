@@ -61,23 +61,31 @@ void launch_spmm_c(const SpmmCArgs& a) {
     })
 }
 
+template <typename TX, typename TO, int CPL, bool VDF, bool NARROW>
+void launch_spmm_a_one(const SpmmAArgs& a) {
+    k_spmm_a<TX, TO, CPL, VDF, NARROW><<<a.blocks, kThreads, 0, a.stream>>>(
+        a.p, static_cast<const TX*>(a.X), static_cast<TO*>(a.out), a.ld, a.sh.L, a.sh.Q, a.v, a.alpha, a.accumulate,
+        a.gate, a.ph);
+}
+
+template <typename TX, typename TO, bool VDF>
+void launch_spmm_a_vdf(const SpmmAArgs& a) {
+    if (a.sh.L <= 2) {
+        launch_spmm_a_one<TX, TO, 1, VDF, true>(a);
+        return;
+    }
+    LORADS_CPL_SWITCH(a.sh.CPL, { launch_spmm_a_one<TX, TO, CPL, VDF, false>(a); })
+}
+
 template <typename TX, typename TO>
 void launch_spmm_a(const SpmmAArgs& a) {
-    const TX* X = static_cast<const TX*>(a.X);
-    TO* out = static_cast<TO*>(a.out);
     if constexpr (!std::is_same_v<arith_t<TO>, double>) {
         if (a.v_df) {
-            LORADS_CPL_SWITCH(a.sh.CPL, {
-                k_spmm_a<TX, TO, CPL, true><<<a.blocks, kThreads, 0, a.stream>>>(
-                    a.p, X, out, a.ld, a.sh.L, a.sh.Q, a.v, a.alpha, a.accumulate, a.gate, a.ph);
-            })
+            launch_spmm_a_vdf<TX, TO, true>(a);
             return;
         }
     }
-    LORADS_CPL_SWITCH(a.sh.CPL, {
-        k_spmm_a<TX, TO, CPL, false><<<a.blocks, kThreads, 0, a.stream>>>(
-            a.p, X, out, a.ld, a.sh.L, a.sh.Q, a.v, a.alpha, a.accumulate, a.gate, a.ph);
-    })
+    launch_spmm_a_vdf<TX, TO, false>(a);
 }
 
 template <typename TU, typename TV>
