@@ -94,6 +94,7 @@ struct Prof {
 
 struct lorads_ctx {
     int64_t n = 0, m = 0, nnz_c = 0, m_diag = 0, m_off = 0, nnz_aoff = 0;
+    RowEntries c_rows{0.0, 0};
     cudaStream_t stream = nullptr;       // caller's stream (entry points)
     cudaStream_t solve_stream = nullptr; // owned, capture-capable
     cudaEvent_t ev_sync = nullptr;
@@ -193,11 +194,11 @@ int row_blocks(const lorads_ctx* c, int64_t rows, int L) {
     return (int)std::min<int64_t>(b, c->max_blocks);
 }
 
-// Fills the grid of a product over C: the tile kernel where a row has one unit per lane.
+// Fills the grid of a product over C, of the tile kernel where that is the faster one.
 // Returns the blocks launched (those whose partial sums the caller folds).
 template <typename TX, typename TO>
 int plan_spmm(const lorads_ctx* c, SpmmCArgs* a) {
-    if (a->sh.Q <= 32) {
+    if (tile_pays<TX, TO>(a->epi, a->v != nullptr && c->pd.dk != nullptr, c->n, a->sh.Q, c->c_rows)) {
         const TilePlan t = tile_plan(c->n, a->sh.Q, c->num_sms * kTileBlocks, tile_threads<TX, TO>());
         a->nsub = t.nsub;
         a->blocks = t.blocks;
@@ -358,6 +359,8 @@ lorads_status validate_and_build(lorads_ctx* ctx, int64_t n, const int64_t* rp, 
     ctx->nnz_aoff = hp.nnz_aoff;
     ctx->n = n; ctx->m = m; ctx->nnz_c = hp.nnz_c; ctx->m_diag = hp.m_diag; ctx->m_off = hp.m_off;
     const int64_t nnz = hp.nnz_c, m_diag = hp.m_diag, m_off = hp.m_off;
+    ctx->c_rows.mean = (double)nnz / (double)n;
+    for (int64_t i = 0; i < n; ++i) ctx->c_rows.longest = std::max(ctx->c_rows.longest, rp[i + 1] - rp[i]);
     // device (queried only once the host-side checks have passed)
     cudaError_t ce = cudaGetDevice(&ctx->device);
     if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);

@@ -34,6 +34,61 @@ inline TilePlan tile_plan(int64_t n, int Q, int most_blocks, int threads) {
     return TilePlan{(int)nsub, (int)(blocks < most_blocks ? blocks : most_blocks)};
 }
 
+// Rows of C: stored entries a row on average, and of the longest row.
+struct RowEntries {
+    double mean;
+    int64_t longest;
+};
+constexpr int kTileInFlight4 = 5, kTileInFlight8 = 4;      // gathers in flight per lane, 4- and 8-byte rows
+
+// Whether the tile kernel is the faster one for a product over C; k_spmm_c takes the others.
+// Both were measured for random graphs of 3 to 20 neighbours a row, lattices of 4 and a dense
+// matrix, n = 1e3 to 1e6, rows of 4 to 128 elements (tile against k_spmm_c, us):
+//  - FP64 line search: everywhere but on long rows (n = 1e6, ld = 20, 4 neighbours: 537 / 1437;
+//    n = 1e3, 500 neighbours, ld = 8: 208 / 193).
+//  - FP64 product: where packed groups keep more lanes busy than groups of a power of two (n = 1e6,
+//    ld = 20, 4 neighbours: 0.74 of the time; ld = 16: 1.0, on a lattice of 1e5 1.1); rows of one
+//    or two units (0.8 to 1.0); long rows not (40 neighbours: 1.06 to 1.16).
+//  - Products in float: on irregular rows a row group waits for the longest of its rows, in rounds
+//    of five gathers, where k_spmm_c has eight in flight (float rows, n = 1e5, ld = 24, 4 neighbours:
+//    30 / 21, 12 neighbours: 51 / 29; dense: 103 / 41).  The tile is faster where every row
+//    takes one round and the streams leave L2 (lattice of 1e6, ld = 20: 98 / 155), and for bf16
+//    rows on up to 12 neighbours, where the weights' FP64 in every lane bounds the other (n = 1e6,
+//    ld = 20, 4 neighbours: 141 / 217; without a multiplier 128 / 148).
+//  - Line search in float: its epilogue gains as in FP64, its gathers lose as above (float rows,
+//    n = 1e6, ld = 24: 0.8 of the time at 3 neighbours, 1.14 at 12).
+template <typename TX, typename TO>
+inline bool tile_pays(int epi, bool weighted, int64_t n, int Q, const RowEntries& c) {
+    if (Q > 32) return false;
+    int L = 1;
+    while (L < Q) L <<= 1;
+    const int busy = 32 / Q * Q, busy_pow2 = 32 / L * Q;   // lanes at work: packed groups, groups of L
+    const bool packed = busy > busy_pow2, by_half = 2 * busy >= 3 * busy_pow2;
+    const double units = (double)n * Q;
+    if (std::is_same_v<arith_t<TO>, dfloat>) return true;  // bound by arithmetic (840 / 355 at n = 1e6)
+    if (std::is_same_v<arith_t<TO>, double>) {
+        if (epi == EPI_LS) return c.mean <= 64;
+        if (c.mean > 24) return false;
+        if (Q <= 2 || packed) return true;
+        if (Q >= 16) return units >= 9e5;
+        if (Q == 4 && n < 50000) return true;
+        return c.mean <= 7.5 && (c.longest > kTileInFlight4 || units >= 1.2e6);
+    }
+    const bool narrow = sizeof(TX) == 2;                   // bf16 rows
+    if (epi == EPI_LS) {
+        if (narrow) return c.mean <= (Q == 1 ? 6 : 22);
+        return Q >= 2 && c.mean <= (Q >= 16 ? 14 : packed ? 10 : 6);
+    }
+    if (c.longest <= kTileInFlight4) {                     // each row in one round of gathers
+        if (narrow) return weighted ? Q >= 2 && units >= 8e5 : Q >= 3 && units >= (packed ? 1.4e6 : 3.5e6);
+        return Q >= 3 && (weighted ? units >= 1.5e6 : packed && units >= 3e6);
+    }
+    if (Q < 3 || units < 3e6) return false;
+    if (!narrow) return weighted && by_half && c.mean <= 4.5;
+    if (weighted) return c.mean <= (by_half ? 13.5 : packed ? 9.5 : 5.5);
+    return packed && c.mean <= (by_half ? 9.5 : 5.5);
+}
+
 // 4 or 8 bytes of global memory to shared memory, without a register.
 template <int BYTES>
 __device__ __forceinline__ void stage_bytes(void* smem, const void* g) {
@@ -76,7 +131,7 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
     using AW = wide_t<TR, TX>;
     using AD = arith_t<TX>;
     constexpr int NW = tile_threads<TX, TO>() / 32;
-    constexpr int UN = sizeof(AD) == 8 ? 4 : 5;            // gathers in flight per lane
+    constexpr int UN = sizeof(AD) == 8 ? kTileInFlight8 : kTileInFlight4;    // gathers in flight per lane
     constexpr bool kSums = EPI == EPI_LS;
     // FP64 line search, bound by the FP64 pipe: a row group takes as many steps as the longest of
     // its rows, so the tile's rows are taken in the order of their lengths, and a tile's p1 and p2
