@@ -724,10 +724,17 @@ struct Driver {
     // iteration each time (five launches); an inner loop that ends within the group leaves the
     // rest of it to return at once.  Four: at n = 1e3 an outer step comes every 20 to 50
     // iterations.  Per iteration, n = 1e3, FP64: 86.5 us with one, 78.7 with four (45 us of it the
-    // control kernels' and the step update's latency).
-    static constexpr int kInnerPerGraph = 4;
+    // control kernels' and the step update's latency).  With inner loops of two iterations a group
+    // of four was still faster (n = 1e3, FP64, 60 iterations: 5.3 ms against 6.2), of one it was not
+    // (600 rows, 9000 constraints, mixed: 9.4 ms against 8.7): no more than an inner loop
+    // may hold, and a divisor of check_every, so that the host polls as often as that says.
+    static int inner_per_graph(const lorads_params& P) {
+        int k = std::min(4, P.max_inner);
+        while (P.check_every % k != 0) --k;
+        return k;
+    }
     void enqueue_iterations() {
-        for (int k = 0; k < kInnerPerGraph; ++k) enqueue_inner();
+        for (int k = inner_per_graph(c->prm); k > 0; --k) enqueue_inner();
         enqueue_outer();
     }
 };
@@ -806,8 +813,10 @@ lorads_status capture(lorads_ctx* ctx) {
         cudaGetLastError();
         return LORADS_ERR_CUDA;
     }
-    e = cudaGraphInstantiate(&st.exec, g, 0);
+    cudaGraphExec_t exec = nullptr;              // the state keeps a graph only once it exists
+    e = cudaGraphInstantiate(&exec, g, 0);
     cudaGraphDestroy(g);
+    if (e == cudaSuccess) st.exec = exec;
     if (e != cudaSuccess) {
         ctx->err = std::string("graph instantiate: ") + cudaGetErrorString(e);
         return LORADS_ERR_CUDA;
@@ -1384,8 +1393,7 @@ lorads_status run_graph(lorads_ctx* ctx, int prec, std::chrono::steady_clock::ti
     // the graph of an earlier solve holds the same kernels and arrays: it is destroyed with the
     // state's arrays, and nothing else that it was captured from changes
     if (!st.exec && (s = capture<TR, TD, TDIR>(ctx))) return s;
-    constexpr int per_graph = Driver<TR, TD, TDIR>::kInnerPerGraph;
-    const int launches = (P.check_every + per_graph - 1) / per_graph;
+    const int launches = P.check_every / Driver<TR, TD, TDIR>::inner_per_graph(P);
     // ---- iterate: launch the graph in batches, poll the status of the previous batch
     int slot = 0;
     bool pending = false;
