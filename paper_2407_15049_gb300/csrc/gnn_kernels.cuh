@@ -123,8 +123,7 @@ k_prep(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ci
             for (int64_t e = rp[i]; e < e1; ++e) {
                 const double w = cv[e];
                 if (ci[e] == i) {
-                    // one stored diagonal entry a row: no FP64 addition to 0 (nor -0 for 0)
-                    dg = (__double_as_longlong(w) << 1) == 0 ? 0.0 : w;
+                    dg += w;
                 } else {
                     deg += 1;
                     s += fabs(w);
