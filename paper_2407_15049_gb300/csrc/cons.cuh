@@ -164,129 +164,106 @@ k_cons_wide(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const T
     CS* zkc = static_cast<CS*>(zk);
     // what each mode gathers besides u_i, u_j
     constexpr bool NEED_V = MODE == CONS_EVAL || MODE == CONS_LS;
-    constexpr int UC = 1;               // constraints in flight per lane group
     RowLoop rl(L, vg);
     const int64_t cnt = k1 - k0;
-    const int64_t step = (int64_t)rl.rows_per_warp;
-    for (int64_t base = rl.first * UC; base < cnt; base += rl.stride * UC) {
-        int64_t t[UC];
-        bool act[UC], diag[UC];
-        int i[UC], j[UC], kid[UC];
-        CS ak[UC], yk[UC], zb[UC];          // coefficient, y_k, and z_k (cached) or b_k
-        Unit<TU> ui[UC][CPL], uj[UC][CPL];
-        Unit<TV> vi[UC][CPL], vj[UC][CPL];
-#pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            t[u] = k0 + base + u * step + rl.gw;
-            act[u] = t[u] < k1;
-            i[u] = act[u] ? __ldg(p.k_row + t[u]) : 0;
-            j[u] = act[u] ? __ldg(p.k_col + t[u]) : 0;
-            if constexpr (MODE == CONS_EVAL || std::is_same_v<CS, double>)
-                ak[u] = act[u] ? CS(__ldg(p.k_a + t[u])) : CS(0.0);
-            else
-                ak[u] = act[u] ? (p.k_adf ? ld_scalar<CS>(p.k_a, p.k_adf, t[u]) : CS(__ldg(p.k_a + t[u]))) : CS(0.0);
-            kid[u] = act[u] ? __ldg(p.k_id + t[u]) : 0;
-            diag[u] = i[u] == j[u];
-        }
-#pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            yk[u] = CS(0.0);
-            zb[u] = CS(0.0);
-            if (!act[u]) continue;
+    for (int64_t base = rl.first; base < cnt; base += rl.stride) {
+        const int64_t t = k0 + base + rl.gw;
+        const bool act = t < k1;
+        const int i = act ? __ldg(p.k_row + t) : 0, j = act ? __ldg(p.k_col + t) : 0;
+        const int k = act ? __ldg(p.k_id + t) : 0;
+        const bool diag = i == j;
+        CS ak = CS(0.0), yk = CS(0.0), zb = CS(0.0);     // coefficient, y_k, and z_k (cached) or b_k
+        Unit<TU> ui[CPL], uj[CPL];
+        Unit<TV> vi[CPL], vj[CPL];
+        if (act) {
+            if constexpr (MODE == CONS_EVAL || std::is_same_v<CS, double>) ak = CS(__ldg(p.k_a + t));
+            else ak = p.k_adf ? ld_scalar<CS>(p.k_a, p.k_adf, t) : CS(__ldg(p.k_a + t));
             if constexpr (MODE != CONS_EVAL) {
-                if constexpr (MODE != CONS_ZZ) {
-                    yk[u] = ld_multiplier<CS>(y, ydf, kid[u]);
-                }
-                if (MODE == CONS_LS && zk != nullptr) zb[u] = zkc[kid[u]];
-                else if constexpr (std::is_same_v<CS, double>) zb[u] = __ldg(p.b + kid[u]);
-                else zb[u] = p.b_df ? ld_scalar<CS>(p.b, p.b_df, kid[u]) : CS(__ldg(p.b + kid[u]));
+                if constexpr (MODE != CONS_ZZ) yk = ld_multiplier<CS>(y, ydf, k);
+                if (MODE == CONS_LS && zk != nullptr) zb = zkc[k];
+                else if constexpr (std::is_same_v<CS, double>) zb = __ldg(p.b + k);
+                else zb = p.b_df ? ld_scalar<CS>(p.b, p.b_df, k) : CS(__ldg(p.b + k));
             }
-            load_row<TU, CPL>(ui[u], U, i[u], ld, L, Q, rl.lig);
-            if (!diag[u]) load_row<TU, CPL>(uj[u], U, j[u], ld, L, Q, rl.lig);
+            load_row<TU, CPL>(ui, U, i, ld, L, Q, rl.lig);
+            if (!diag) load_row<TU, CPL>(uj, U, j, ld, L, Q, rl.lig);
             if constexpr (NEED_V) {
                 if (!(MODE == CONS_EVAL && same)) {
-                    load_row<TV, CPL>(vi[u], V, i[u], ld, L, Q, rl.lig);
-                    if (!diag[u]) load_row<TV, CPL>(vj[u], V, j[u], ld, L, Q, rl.lig);
+                    load_row<TV, CPL>(vi, V, i, ld, L, Q, rl.lig);
+                    if (!diag) load_row<TV, CPL>(vj, V, j, ld, L, Q, rl.lig);
                 }
             }
         }
-#pragma unroll
-        for (int u = 0; u < UC; ++u) {
-            // dots of the gathered rows; partial per lane, then group sums
-            AU s_uu = AU(0);                  // u_i.u_j (EVAL with U==V, and R-only modes)
-            AW s_uv = AW(0), s_vu = AW(0);    // u_i.v_j, u_j.v_i
-            AV s_vv = AV(0);                  // v_i.v_j
-            if (act[u]) {
-                if constexpr (MODE == CONS_EVAL) {
-                    if (same) {
-                        s_uu = diag[u] ? dot_units<AU>(ui[u], ui[u]) : dot_units<AU>(ui[u], uj[u]);
-                    } else if (diag[u]) {
-                        s_uv = dot_units<AW>(ui[u], vi[u]);
-                    } else {
-                        s_uv = dot_units<AW>(ui[u], vj[u]);
-                        s_vu = dot_units<AW>(uj[u], vi[u]);
-                    }
+        // dots of the gathered rows; partial per lane, then group sums
+        AU s_uu = AU(0);                  // u_i.u_j (EVAL with U==V, and R-only modes)
+        AW s_uv = AW(0), s_vu = AW(0);    // u_i.v_j, u_j.v_i
+        AV s_vv = AV(0);                  // v_i.v_j
+        if (act) {
+            if constexpr (MODE == CONS_EVAL) {
+                if (same) {
+                    s_uu = diag ? dot_units<AU>(ui, ui) : dot_units<AU>(ui, uj);
+                } else if (diag) {
+                    s_uv = dot_units<AW>(ui, vi);
                 } else {
-                    if (MODE != CONS_LS || zk == nullptr)
-                        s_uu = diag[u] ? dot_units<AU>(ui[u], ui[u]) : dot_units<AU>(ui[u], uj[u]);
-                    if constexpr (MODE == CONS_LS) {
-                        if (diag[u]) {
-                            s_uv = dot_units<AW>(ui[u], vi[u]);
-                            s_vu = s_uv;
-                            s_vv = dot_units<AV>(vi[u], vi[u]);
-                        } else {
-                            s_uv = dot_units<AW>(ui[u], vj[u]);
-                            s_vu = dot_units<AW>(vi[u], uj[u]);
-                            s_vv = dot_units<AV>(vi[u], vj[u]);
-                        }
+                    s_uv = dot_units<AW>(ui, vj);
+                    s_vu = dot_units<AW>(uj, vi);
+                }
+            } else {
+                if (MODE != CONS_LS || zk == nullptr) s_uu = diag ? dot_units<AU>(ui, ui) : dot_units<AU>(ui, uj);
+                if constexpr (MODE == CONS_LS) {
+                    if (diag) {
+                        s_uv = dot_units<AW>(ui, vi);
+                        s_vu = s_uv;
+                        s_vv = dot_units<AV>(vi, vi);
+                    } else {
+                        s_uv = dot_units<AW>(ui, vj);
+                        s_vu = dot_units<AW>(vi, uj);
+                        s_vv = dot_units<AV>(vi, vj);
                     }
                 }
             }
-            s_uu = group_sum(s_uu, L);
-            if constexpr (MODE == CONS_EVAL || MODE == CONS_LS) {
-                s_uv = group_sum(s_uv, L);
-                s_vu = group_sum(s_vu, L);
-                s_vv = group_sum(s_vv, L);
-            }
-            if (act[u] && rl.lig == 0) {
-                const int k = kid[u];
-                if constexpr (MODE == CONS_EVAL) {
-                    const double a = double(ak[u]);
-                    const double f = diag[u] ? 1.0 : 2.0;
-                    double val;
-                    if (same) val = f * a * double(s_uu);
-                    else if (diag[u]) val = a * double(s_uv);
-                    else val = a * (double(s_uv) + double(s_vu));
-                    static_cast<double*>(out)[k] = val;
-                } else {
-                    const CS fa = diag[u] ? ak[u] : CS(2.0f) * ak[u];
-                    const CS z = (MODE == CONS_LS && zk != nullptr) ? zb[u] : fa * CS(s_uu) - zb[u];
-                    if constexpr (MODE == CONS_LS) {
-                        const CS yt = yk[u] - rho_c * z;
-                        const CS q1 = fa * (CS(s_uv) + CS(s_vu));
-                        const CS q2 = fa * CS(s_vv);
-                        accq[PL_YQ1] += PA(yt * q1);
-                        accq[PL_YQ2] += PA(yt * q2);
-                        accq[PL_Q1Q1] += PA(q1 * q1);
-                        accq[PL_Q1Q2] += PA(q1 * q2);
-                        accq[PL_Q2Q2] += PA(q2 * q2);
+        }
+        s_uu = group_sum(s_uu, L);
+        if constexpr (NEED_V) {
+            s_uv = group_sum(s_uv, L);
+            s_vu = group_sum(s_vu, L);
+            s_vv = group_sum(s_vv, L);
+        }
+        if (!act || rl.lig != 0) continue;
+        if constexpr (MODE == CONS_EVAL) {
+            const double a = double(ak);
+            const double f = diag ? 1.0 : 2.0;
+            double val;
+            if (same) val = f * a * double(s_uu);
+            else if (diag) val = a * double(s_uv);
+            else val = a * (double(s_uv) + double(s_vu));
+            static_cast<double*>(out)[k] = val;
+        } else {
+            const CS fa = diag ? ak : CS(2.0f) * ak;
+            const CS z = (MODE == CONS_LS && zk != nullptr) ? zb : fa * CS(s_uu) - zb;
+            if constexpr (MODE == CONS_LS) {
+                const CS yt = yk - rho_c * z;
+                const CS q1 = fa * (CS(s_uv) + CS(s_vu));
+                const CS q2 = fa * CS(s_vv);
+                accq[PL_YQ1] += PA(yt * q1);
+                accq[PL_YQ2] += PA(yt * q2);
+                accq[PL_Q1Q1] += PA(q1 * q1);
+                accq[PL_Q1Q2] += PA(q1 * q2);
+                accq[PL_Q2Q2] += PA(q2 * q2);
+            } else {
+                accq[PC_ZZ] += PA(z * z);
+                if constexpr (MODE == CONS_YTIL) {
+                    static_cast<CS*>(out)[k] = yk - rho_c * z;
+                    if (zk != nullptr) zkc[k] = z;
+                } else if constexpr (MODE == CONS_YUPD) {
+                    const CS yn = yk - rho_c * z;
+                    y[k] = double(yn);
+                    if constexpr (std::is_same_v<CS, dfloat>) {
+                        if (ydf != nullptr) ydf[k] = yn;
                     } else {
-                        accq[PC_ZZ] += PA(z * z);
-                        if constexpr (MODE == CONS_YTIL) {
-                            static_cast<CS*>(out)[k] = yk[u] - rho_c * z;
-                            if (zk != nullptr) zkc[k] = z;
-                        } else if constexpr (MODE == CONS_YUPD) {
-                            const CS yn = yk[u] - rho_c * z;
-                            y[k] = double(yn);
-                            if constexpr (std::is_same_v<CS, dfloat>) {
-                                if (ydf != nullptr) ydf[k] = yn;
-                            } else {
-                                if (ydf != nullptr) ydf[k] = dfloat(yn);
-                            }
-                            // b_k: zb holds it (z is recomputed in this mode)
-                            accq[PC_BY] += PA(zb[u] * yn);
-                        }
+                        if (ydf != nullptr) ydf[k] = dfloat(yn);
                     }
+                    // b_k: zb holds it (z is recomputed in this mode)
+                    accq[PC_BY] += PA(zb * yn);
                 }
             }
         }

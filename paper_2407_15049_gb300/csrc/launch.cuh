@@ -33,13 +33,21 @@ void launch_spmm_tile(const SpmmCArgs& a) {
 }
 
 // The line-search form takes the prefetch depth (and packed groups) as template
-// arguments; the other epilogues run without prefetch.
+// arguments; the other epilogues run without prefetch.  What each type is asked for: the plain
+// product and the line search without a cache of z (both forms of the kernel) by the standalone
+// calls, whose R is not double-float; the objective by the solves, whose three types are then
+// the same (in double-float by the tile kernel alone where a row has one unit a lane).
 template <typename TX, typename TO, typename TR>
 void launch_spmm_c(const SpmmCArgs& a) {
+    constexpr bool kStandalone = !std::is_same_v<TR, dfloat>;
+    constexpr bool kObjective = std::is_same_v<TX, TO> && std::is_same_v<TX, TR>;
     if (a.nsub > 0) {
-        if (a.epi == EPI_LS) launch_spmm_tile<TX, TO, TR, EPI_LS>(a);
-        else if (a.epi == EPI_OBJ) launch_spmm_tile<TX, TO, TR, EPI_OBJ>(a);
-        else launch_spmm_tile<TX, TO, TR, EPI_NONE>(a);
+        if constexpr (kObjective)
+            if (a.epi == EPI_OBJ) launch_spmm_tile<TX, TO, TR, EPI_OBJ>(a);
+        if constexpr (kStandalone) {
+            if (a.epi == EPI_LS) launch_spmm_tile<TX, TO, TR, EPI_LS>(a);
+            else if (a.epi == EPI_NONE) launch_spmm_tile<TX, TO, TR, EPI_NONE>(a);
+        }
         return;
     }
     if (a.epi == EPI_LS && a.dense && packed_rows_gain(a.sh)) {
@@ -54,9 +62,10 @@ void launch_spmm_c(const SpmmCArgs& a) {
             else if (a.prefetch == 1) launch_spmm_c_one<TX, TO, TR, CPL, EPI_LS, false, 1>(a, a.sh.L);
             else launch_spmm_c_one<TX, TO, TR, CPL, EPI_LS, false, 0>(a, a.sh.L);
         } else if (a.epi == EPI_OBJ) {
-            launch_spmm_c_one<TX, TO, TR, CPL, EPI_OBJ, false, 0>(a, a.sh.L);
+            if constexpr (kObjective && (CPL > 1 || kStandalone))
+                launch_spmm_c_one<TX, TO, TR, CPL, EPI_OBJ, false, 0>(a, a.sh.L);
         } else {
-            launch_spmm_c_one<TX, TO, TR, CPL, EPI_NONE, false, 0>(a, a.sh.L);
+            if constexpr (kStandalone) launch_spmm_c_one<TX, TO, TR, CPL, EPI_NONE, false, 0>(a, a.sh.L);
         }
     })
 }
