@@ -762,25 +762,32 @@ lorads_status alloc_state(lorads_ctx* ctx, int prec, int r) {
     st.esDir = sizeof(TDIR);
     st.rtype = std::is_same<TR, double>::value ? 0 : (std::is_same<TR, dfloat>::value ? 1 : 2);
     const size_t nl = (size_t)ctx->n * ld;
-    lorads_status s;
     const int T = ctx->prm.lbfgs_mem;
-    if ((s = dalloc(ctx, reinterpret_cast<TR**>(&st.R), nl))) return s;
-    if ((s = dalloc(ctx, reinterpret_cast<TR**>(&st.CR), nl))) return s;
-    if ((s = dalloc(ctx, reinterpret_cast<TDIR**>(&st.D), nl))) return s;
-    if ((s = dalloc(ctx, reinterpret_cast<TD**>(&st.CD), nl))) return s;
-    if ((s = dalloc(ctx, reinterpret_cast<TD**>(&st.G), nl))) return s;
-    if ((s = dalloc(ctx, reinterpret_cast<TDIR**>(&st.hist), nl * 2 * T))) return s;
-    st.slot_stride = (int64_t)nl;
-    if (ctx->m_off) {
-        if ((s = dalloc(ctx, reinterpret_cast<TD**>(&st.W), nl))) return s;
-        if ((s = dalloc(ctx, &st.ytil, ctx->m))) return s;
-    }
-    if ((s = dalloc(ctx, &st.y, ctx->m))) return s;
     const bool fp64_path = std::is_same<TR, double>::value && std::is_same<TD, double>::value;
-    // z cache: double (FP64), double-float (DF64) or float (mixed, FP32): 8 bytes covers all
-    if ((s = dalloc(ctx, reinterpret_cast<double**>(&st.zrow), ctx->n))) return s;
-    if (!fp64_path && (s = dalloc(ctx, &st.ydf, ctx->m))) return s;
-    if ((s = dalloc(ctx, &st.zk, ctx->m))) return s;
+    auto arrays = [&]() -> lorads_status {
+        lorads_status s;
+        if ((s = dalloc(ctx, reinterpret_cast<TR**>(&st.R), nl))) return s;
+        if ((s = dalloc(ctx, reinterpret_cast<TR**>(&st.CR), nl))) return s;
+        if ((s = dalloc(ctx, reinterpret_cast<TDIR**>(&st.D), nl))) return s;
+        if ((s = dalloc(ctx, reinterpret_cast<TD**>(&st.CD), nl))) return s;
+        if ((s = dalloc(ctx, reinterpret_cast<TD**>(&st.G), nl))) return s;
+        if ((s = dalloc(ctx, reinterpret_cast<TDIR**>(&st.hist), nl * 2 * T))) return s;
+        st.slot_stride = (int64_t)nl;
+        if (ctx->m_off) {
+            if ((s = dalloc(ctx, reinterpret_cast<TD**>(&st.W), nl))) return s;
+            if ((s = dalloc(ctx, &st.ytil, ctx->m))) return s;
+        }
+        if ((s = dalloc(ctx, &st.y, ctx->m))) return s;
+        // z cache: double (FP64), double-float (DF64) or float (mixed, FP32): 8 bytes covers all
+        if ((s = dalloc(ctx, reinterpret_cast<double**>(&st.zrow), ctx->n))) return s;
+        if (!fp64_path && (s = dalloc(ctx, &st.ydf, ctx->m))) return s;
+        return dalloc(ctx, &st.zk, ctx->m);
+    };
+    const lorads_status s = arrays();
+    if (s != LORADS_OK) {
+        free_state(st);                             // no later call takes a part of a state for a whole one
+        return s;
+    }
     // cleared on the stream that fills and reads them: it does not wait for the default stream
     cudaStream_t ss = ctx->solve_stream;
     CK(cudaMemsetAsync(st.R, 0, nl * sizeof(TR), ss));
