@@ -271,12 +271,22 @@ k_cons_wide(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const T
     if constexpr (MODE != CONS_EVAL) block_partials<NQ>(accq, part, vg.pslot);
 }
 
-// Per-lane partial dot of gathered rows, by the arithmetic type's own multiply-add.
+// Per-lane partial dot of gathered rows, by the arithmetic type's own multiply-add; a double-float
+// row with a float row by the product of a double word and a float, which drops the terms of the
+// zero low parts.
+template <typename T1, typename T2>
+constexpr bool df_by_float() {
+    return std::is_same_v<arith_t<T1>, dfloat> && std::is_same_v<arith_t<T2>, float>;
+}
 template <typename A, typename T1, typename T2>
 __device__ __forceinline__ A dot_lane(const Unit<T1>& x, const Unit<T2>& y) {
     A s = A(0);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) s = fma(A(x.v[e]), A(y.v[e]), s);
+    for (int e = 0; e < 4; ++e) {
+        if constexpr (df_by_float<T1, T2>()) s = mul_fp(x.v[e], y.v[e]) + s;
+        else if constexpr (df_by_float<T2, T1>()) s = mul_fp(y.v[e], x.v[e]) + s;
+        else s = fma(A(x.v[e]), A(y.v[e]), s);
+    }
     return s;
 }
 
@@ -411,7 +421,10 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
         // ---- dots of the group's constraints
         AU s_z[kConsBatch];                  // u_i.u_j (R-only modes, EVAL with U == V)
         // u_i.v_j and u_j.v_i apart: rounded sums of a float dot each, added in CS (in one float
-        // chain q1 lost a fifth: rms 1.41e-8 -> 1.68e-8 at r = 20)
+        // chain q1 lost a fifth: rms 1.41e-8 -> 1.68e-8 at r = 20).  With double-float rows and a
+        // float direction the lanes' dots are added first: emulated at r = 20 the rms error is
+        // 3.49e-16, and 3.60e-16 with a sum of each over the lanes and general products.
+        constexpr bool kOneSum = MODE == CONS_LS && df_by_float<TU, TV>();
         AW s_1[kConsBatch], s_1b[kConsBatch];
         AV s_2[kConsBatch];                  // v_i.v_j
 #pragma unroll
@@ -457,6 +470,7 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
                     if constexpr (MODE == CONS_LS) {
                         s_1[u0 + c] = dot_lane<AW>(ui[c][0], vj[c][0]);
                         s_1b[u0 + c] = dot_lane<AW>(vi[c][0], uj[c][0]);
+                        if constexpr (kOneSum) s_1[u0 + c] = s_1[u0 + c] + s_1b[u0 + c];
                         s_2[u0 + c] = dot_lane<AV>(vi[c][0], vj[c][0]);
                     }
                 }
@@ -473,7 +487,7 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
             if constexpr (NEED_Z) batch_sums(s_z, L, rl.lig);
             if constexpr (MODE == CONS_LS) {
                 batch_sums(s_1, L, rl.lig);
-                batch_sums(s_1b, L, rl.lig);
+                if constexpr (!kOneSum) batch_sums(s_1b, L, rl.lig);
                 batch_sums(s_2, L, rl.lig);
             }
         }
@@ -494,7 +508,9 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
             else z = fa * CS(s_z[0]) - zb;
             if constexpr (MODE == CONS_LS) {
                 const CS yt = yk - rho_c * z;
-                const CS q1 = fa * (CS(s_1[0]) + CS(s_1b[0]));
+                CS q1;
+                if constexpr (kOneSum) q1 = fa * CS(s_1[0]);
+                else q1 = fa * (CS(s_1[0]) + CS(s_1b[0]));
                 const CS q2 = fa * CS(s_2[0]);
                 accq[PL_YQ1] += PA(yt * q1);
                 accq[PL_YQ2] += PA(yt * q2);

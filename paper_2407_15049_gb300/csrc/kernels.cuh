@@ -300,7 +300,10 @@ __device__ __forceinline__ A_of_t<TO> spmm_a_weight(const ProbDev& p, const void
 }
 
 // acc += the weighted rows of the slots [s, s1), four slots in flight, each weight formed by
-// every lane.  For groups of one and two lanes, which have little to share.
+// every lane.  For groups of one and two lanes, which have little to share and, with a slot a
+// lane as the wider groups take them, one or two rows in flight (product of 4e5 constraints on 2e4
+// rows, v double, us here and with a slot a lane: FP64, ld = 4, 49 and 102, ld = 8, 64 and 91; bf16,
+// ld = 4, 33 and 64; 1000 x 60000, FP64, ld = 4: 196 and 500).
 template <typename TX, typename TO, int CPL, bool VDF>
 __device__ __forceinline__ void
 spmm_a_row_narrow(const ProbDev& p, const TX* __restrict__ X, int ld, int L, int Q, const void* __restrict__ v,
@@ -352,7 +355,10 @@ k_spmm_a_body(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld,
     // products and a conversion per slot and lane).
     const int B = L < 8 ? L : 8;
     constexpr int UN = CPL == 1 ? (sizeof(TX) == 8 ? 4 : 8) : 2;     // rows in flight per lane
-    // bf16 rows: a slot past the end loads a row of zeros under a mask in place of a branch
+    // bf16 rows: a slot past the end loads a row of zeros under a mask; with a branch around each
+    // load they were not in flight together (5.4e6 slots on 1e5 rows, ld = 24: 190 and 109 us; 1000 x
+    // 60000, ld = 16: 141 and 95, where four slots in every lane took 116).  The 4- and 8-byte
+    // rows keep the branch: FP64 1000 x 60000, ld = 16: 152, 172 under the mask.
     constexpr bool kMasked = sizeof(TX) == 2;
     for (int64_t base = rl.first; base < p.n; base += rl.stride) {
         const int64_t i = base + rl.gw;
