@@ -421,10 +421,11 @@ k_cons_batch(ProbDev p, int64_t k0, int64_t k1, const TU* __restrict__ U, const 
         // ---- dots of the group's constraints
         AU s_z[kConsBatch];                  // u_i.u_j (R-only modes, EVAL with U == V)
         // u_i.v_j and u_j.v_i apart: rounded sums of a float dot each, added in CS (in one float
-        // chain q1 lost a fifth: rms 1.41e-8 -> 1.68e-8 at r = 20).  With double-float rows and a
-        // float direction the lanes' dots are added first: emulated at r = 20 the rms error is
-        // 3.49e-16, and 3.60e-16 with a sum of each over the lanes and general products.
-        constexpr bool kOneSum = MODE == CONS_LS && df_by_float<TU, TV>();
+        // chain q1 lost a fifth: rms 1.41e-8 -> 1.68e-8 at r = 20).  In FP64, and with double-float
+        // rows and a float direction, CS adds no bits and the lanes' dots are added first: in
+        // emulation the rms error of FP64 is the same within its noise, that of the mixed form
+        // 3.49e-16 at r = 20 against 3.60e-16 with a sum of each and general products.
+        constexpr bool kOneSum = MODE == CONS_LS && (std::is_same_v<AW, double> || df_by_float<TU, TV>());
         AW s_1[kConsBatch], s_1b[kConsBatch];
         AV s_2[kConsBatch];                  // v_i.v_j
 #pragma unroll

@@ -48,7 +48,8 @@ constexpr int kTileInFlight4 = 5, kTileInFlight8 = 4;      // gathers in flight 
 //    n = 1e3, 500 neighbours, ld = 8: 208 / 193).
 //  - FP64 product: where packed groups keep more lanes busy than groups of a power of two (n = 1e6,
 //    ld = 20, 4 neighbours: 0.74 of the time; ld = 16: 1.0, on a lattice of 1e5 1.1); rows of one
-//    or two units (0.8 to 1.0); long rows not (40 neighbours: 1.06 to 1.16).
+//    or two units (0.8 to 1.0), rows of up to three entries (C = I, n = 5e4: 0.55 to 0.8); long
+//    rows not (40 neighbours: 1.06 to 1.16).
 //  - Products in float: on irregular rows a row group waits for the longest of its rows, in rounds
 //    of five gathers, where k_spmm_c has eight in flight (float rows, n = 1e5, ld = 24, 4 neighbours:
 //    30 / 21, 12 neighbours: 51 / 29; dense: 103 / 41).  The tile is faster where every row
@@ -69,7 +70,7 @@ inline bool tile_pays(int epi, bool weighted, int64_t n, int Q, const RowEntries
     if (std::is_same_v<arith_t<TO>, double>) {
         if (epi == EPI_LS) return c.mean <= 64;
         if (c.mean > 24) return false;
-        if (Q <= 2 || packed) return true;
+        if (Q <= 2 || packed || c.mean <= 3.5) return true;
         if (Q >= 16) return units >= 9e5;
         if (Q == 4 && n < 50000) return true;
         return c.mean <= 7.5 && (c.longest > kTileInFlight4 || units >= 1.2e6);
@@ -80,6 +81,7 @@ inline bool tile_pays(int epi, bool weighted, int64_t n, int Q, const RowEntries
         return Q >= 2 && c.mean <= (Q >= 16 ? 14 : packed ? 10 : 6);
     }
     if (c.longest <= kTileInFlight4) {                     // each row in one round of gathers
+        if (c.mean <= 3.5 && (packed || units <= 1e5 || (narrow && Q > 1))) return true;
         if (narrow) return weighted ? Q >= 2 && units >= 8e5 : Q >= 3 && units >= (packed ? 1.4e6 : 3.5e6);
         return Q >= 3 && (weighted ? units >= 1.5e6 : packed && units >= 3e6);
     }
@@ -98,6 +100,22 @@ __device__ __forceinline__ void stage_bytes(void* smem, const void* g) {
 __device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Sum of a row's Q values in shared memory by one lane, as group_sum adds the values of L >= Q lanes
+// (zeros past Q): at the last exchange the even and the odd lanes meet, at the first l and l + L/2.
+template <int L, int OFF, int STEP, typename V>
+__device__ __forceinline__ V row_tree_part(const V* s, int Q) {
+    if constexpr (STEP >= L) return OFF < Q ? s[OFF] : V(0);
+    else return row_tree_part<L, OFF, 2 * STEP>(s, Q) + row_tree_part<L, OFF + STEP, 2 * STEP>(s, Q);
+}
+template <typename V>
+__device__ __forceinline__ V row_tree(const V* s, int Q) {
+    if (Q <= 2) return row_tree_part<2, 0, 1>(s, Q);
+    if (Q <= 4) return row_tree_part<4, 0, 1>(s, Q);
+    if (Q <= 8) return row_tree_part<8, 0, 1>(s, Q);
+    if (Q <= 16) return row_tree_part<16, 0, 1>(s, Q);
+    return row_tree_part<32, 0, 1>(s, Q);
+}
 
 // out = C X (- A*_diag(v) X), EPI as in k_spmm_c (kernels.cuh); EPI_LS without a cache of z (the
 // line search of a caller's own method).  Why tiles: with one row group at a time every lane of
@@ -320,17 +338,10 @@ k_spmm_tile(ProbDev p, const TX* __restrict__ X, TO* __restrict__ out, int ld, i
         }
         if constexpr (EPI == EPI_LS) {
             if (kc >= 0) {
-                // the tree of group_sum over the row's lanes (a chain of up to 32 would round more)
-                AD *rd = s_rd[wib] + lane * Q, *dd = s_dd[wib] + lane * Q;
-                AW* rr = s_rr[wib] + lane * Q;
-                for (int h = Q > 1 ? 1 << (31 - __clz(Q - 1)) : 0; h > 0; h >>= 1)
-                    for (int q = 0; q < h && q + h < Q; ++q) {
-                        rd[q] += rd[q + h];
-                        dd[q] += dd[q + h];
-                        rr[q] += rr[q + h];
-                    }
-                const AD t_rd = rd[0], t_dd = dd[0];
-                const AW t_rr = rr[0];
+                // (a chain of up to 32 additions would round more than the groups' tree)
+                const AD t_rd = row_tree(s_rd[wib] + lane * Q, Q);
+                const AD t_dd = row_tree(s_dd[wib] + lane * Q, Q);
+                const AW t_rr = row_tree(s_rr[wib] + lane * Q, Q);
                 LS a, z, yv;
                 if constexpr (std::is_same_v<LS, double>) {
                     a = __ldg(p.da + my);
