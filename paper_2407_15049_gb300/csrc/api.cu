@@ -77,6 +77,7 @@ struct AdmmState {
 // Per-kernel-family CUDA-event timing of the host-stepped (verbose >= 2) solve.
 enum { FAM_DIR = 0, FAM_SPMM_LS, FAM_CONS_LS, FAM_ROOT, FAM_STEP, FAM_CONS_YTIL, FAM_SPMM_A, FAM_UPDATE, FAM_HIST,
        FAM_CONS_YUPD, FAM_SPMM_CR, FAM_OUTER, FAM_GRAD, FAM_MISC, NFAM };
+// (k_spmm_c(CR,obj): the product C R in whichever kernel it takes)
 const char* const kFamNames[NFAM] = {"k_dir", "k_spmm_c(CD,ls)", "k_cons(ls)", "k_ctrl_root", "k_step",
                                      "k_cons(ytil)", "k_spmm_a", "k_update(step)", "k_ctrl_hist",
                                      "k_cons(yupd)", "k_spmm_c(CR,obj)", "k_ctrl_outer", "k_update(grad)",

@@ -230,12 +230,14 @@ __device__ __forceinline__ void gather_row(int64_t i, bool act, const int64_t* _
 }
 
 // ------------------------------------------------------------------ forward layer
-// m = aggregate(in), h = relu(W_s in + W_n m + b) for a warp's tile of 16 nodes; OUT: also
-// o = W_o h + b_o, r_hat = o / ||o||.  m and h are stored only where the caller keeps them
+// m = aggregate(in), h = relu(W_s in + W_n m + b) for a warp's tile of kFwdTile = 8 nodes; OUT:
+// also o = W_o h + b_o, r_hat = o / ||o||.  m and h are stored only where the caller keeps them
 // (the backward pass, the next layer); the tile's rows stay in shared memory between the
-// three parts.  A thread owns 4 outputs of 4 nodes: per 4 inputs it reads 16 vectors of
-// shared memory for 128 multiply-adds (one weight and one activation for each multiply-add,
-// with an 8-way bank conflict on the weights, took 1.45 ms a layer at n = 1e6 and the aggregation before it 0.18; now 0.22 together, 0.35 with the output layer).
+// three parts.  A thread owns 4 outputs of kFwdNodes = 2 nodes: per 4 inputs it reads 12 vectors
+// of shared memory for 64 multiply-adds, and shared memory is what bounds it (66 to 71% busy; one
+// weight and one activation for each multiply-add, with an 8-way bank conflict on the weights,
+// took 1.45 ms a layer at n = 1e6 and the aggregation before it 0.18; now 0.23 together, 0.36
+// with the output layer; 4 nodes a thread took 0.33 to 0.60 with fewer warps).
 // Every sum keeps its order: input by input, W_n m before W_s h.
 template <typename TA, int F, bool OUT>
 __global__ void __launch_bounds__(kFwdThreads, kFwdBlocks)

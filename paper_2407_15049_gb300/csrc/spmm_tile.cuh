@@ -9,7 +9,10 @@
 namespace lorads {
 
 constexpr int kTileLaneRows = 192;        // row sums of a tile: rows x Q partials at most
-constexpr int kTileEntries = 160;         // stored entries of a tile held in shared memory
+// Stored entries of a tile held in shared memory.  A tile of 30 rows (n >= 3e5, ld = 20) holds more
+// from 4.3 neighbours a row on, and reads them from global memory; the FP64 line search is still
+// the faster form there (12 neighbours: 0.47 of k_spmm_c's time).
+constexpr int kTileEntries = 160;
 
 // Threads per block: 8-byte forms take twice the shared memory a warp.
 template <typename TX, typename TO> constexpr int tile_threads() {
@@ -44,7 +47,7 @@ constexpr int kTileInFlight4 = 5, kTileInFlight8 = 4;      // gathers in flight 
 // Whether the tile kernel is the faster one for a product over C; k_spmm_c takes the others.
 // Both were measured for random graphs of 3 to 20 neighbours a row, lattices of 4 and a dense
 // matrix, n = 1e3 to 1e6, rows of 4 to 128 elements (tile against k_spmm_c, us):
-//  - FP64 line search: everywhere but on long rows (n = 1e6, ld = 20, 4 neighbours: 537 / 1437;
+//  - FP64 line search: everywhere but on long rows (n = 1e6, ld = 20, 4 neighbours: 545 / 1437;
 //    n = 1e3, 500 neighbours, ld = 8: 208 / 193).
 //  - FP64 product: where packed groups keep more lanes busy than groups of a power of two (n = 1e6,
 //    ld = 20, 4 neighbours: 0.74 of the time; ld = 16: 1.0, on a lattice of 1e5 1.1); rows of one
@@ -144,9 +147,9 @@ __device__ __forceinline__ V row_tree(V* s, int Q) {
 //    is computed, so that a row's gathers wait on no index load;
 //  - the row sums go through shared memory and are taken by lane = row.
 // Element sums keep the order of the stored entries.  Measured: line search in FP64, n = 1e6,
-// ld = 20, 5e6 entries: 1437 -> 537 us, 631 before the rows were sorted and its sums
-// fused (346 us of FP64 multiply-adds at two lanes a cycle);
-// double-float C R with the objective, n = 1e6, ld = 24: 840 -> 355 us; float product with a
+// ld = 20, 5e6 entries: 1437 -> 545 us, 631 before the rows were sorted and a tile's sums
+// fused (346 us of FP64 multiply-adds at two lanes a cycle; the FP64 pipe is 89% busy);
+// double-float C R with the objective, n = 1e6, ld = 24: 840 -> 360 us; float product with a
 // multiplier on a 1000 x 1000 torus, ld = 20: 146 -> 121 us with eight gathers in flight a lane and
 // 3 blocks per SM, 89 us with five and 4 (four: 96 us).  The line search of the solve keeps
 // k_spmm_c: its scalars are few in float, and the tile form took 318 us (24 resident warps) where
